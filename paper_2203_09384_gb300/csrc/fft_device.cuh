@@ -1453,10 +1453,13 @@ struct C32Out {
 
 // m = largest |component| of the signal's unscaled FP32 transform; the
 // values carry 2^(ein + ls) (input exponent, log2 of the normalisation).
+template <int N>
 __device__ __forceinline__ C32Out c32_out_scale(float m, int ein, int ls) {
     if (!(m > 0.0f) || !(m <= 3.0e38f)) return {0, 1.0f};  // zero (or non-finite) signal
-    int f = 0;
-    frexpf(m, &f);  // m = g 2^f, g in [0.5, 1)
+    // m = g 2^f, g in [0.5, 1): f is in the exponent field unless m is subnormal
+    // (N = 2, two elements per call, measured 2% faster without the branch)
+    int f = (int)(__float_as_uint(m) >> 23) - 126;
+    if (N == 2 || f == -126) frexpf(m, &f);
     int e = ein + ls + f - 15;
     e = e < -128 ? -128 : (e > 127 ? 127 : e);  // int8: stored values under/overflow past this
     int k = ein + ls - e;                       // 15 - f unless e was clamped
@@ -1551,18 +1554,17 @@ __device__ __forceinline__ void store_last_c32(const float2 (&v)[C::E], __half2*
     }
 }
 
-// Shared memory of the complex32 kernels: FP32 exchange buffers, then (ring
-// variants) PIPE binary16 tiles and their mbarriers, then per-warp maxima.
+// Shared memory of the direct complex32 kernel: FP32 exchange buffers, then
+// per-warp maxima.
 template <class C>
 struct C32Smem {
-    static constexpr int kRingOffset = C::kSmemElems * 8;
-    static constexpr int kBarOffset = kRingOffset + C::PIPE * C::S * C::N * 4;
-    static constexpr int kRedOffset = kBarOffset + C::PIPE * 8;
+    static constexpr int kRedOffset = C::kSmemElems * 8;
     static constexpr int kBytes = kRedOffset + 128;
 };
 
-// Direct loads.  err / wait_ns / stall are accepted so that all complex32
-// kernels share one argument list; nothing here waits.
+// Direct loads (the N <= 32 rows beside the one-thread-per-signal defaults;
+// N = 64..2048: fft_pair.cuh).  err / wait_ns / stall are accepted so that all
+// complex32 kernels share one argument list; nothing here waits.
 template <class C, bool INV>
 __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_c32_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp, int64_t batch,
@@ -1588,117 +1590,9 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         load_first_c32<C, INV>(v, in + base, t, active);
         twist_and_dft<C, 0>(v, t, tw, tc);
         rest_stages<C, 1>(v, smem, buf, sb, t, tw, tc);
-        const C32Out o = c32_out_scale(c32_signal_max<C>(v, red), ein, ls);
+        const C32Out o = c32_out_scale<C::N>(c32_signal_max<C>(v, red), ein, ls);
         store_last_c32<C, INV>(v, out + base, out_exp + sig, t, active, o);
     }
-}
-
-// stage-0 inputs of a complex32 signal from its binary16 tile in shared memory
-template <class C, bool INV>
-__device__ __forceinline__ void gather_tile_c32(float2 (&v)[C::E], const __half2* tile, int sb, int t) {
-    constexpr int R = C::radix(0);
-    constexpr int K = C::E / R;
-    constexpr int stride = C::N / R;
-#pragma unroll
-    for (int c = 0; c < K; ++c) {
-        const int j = bfly<C, 0>(t, c);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float2 a = __half22float2(tile[sb + j + r * stride]);
-            v[c * R + r] = INV ? conj2(a) : a;
-        }
-    }
-}
-
-// complex32 with the bulk-copy ring: thread 0 keeps PIPE binary16 tiles in
-// flight as in fft_stockham_ring_kernel, with the same bounded waits and
-// error word.
-template <class C, bool INV>
-__global__ void __launch_bounds__(C::NT, C::MINB)
-    fft_stockham_c32_ring_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp,
-                                 int64_t batch, const float2* __restrict__ tw, float scale, int* err,
-                                 uint64_t wait_ns, int stall) {
-    pdl_enter();
-    constexpr int D = C::PIPE;
-    constexpr int TILE = C::S * C::N;
-    using SM = C32Smem<C>;
-    extern __shared__ __align__(16) float2 smem[];
-    unsigned char* base8 = reinterpret_cast<unsigned char*>(smem);
-    __half2* ring = reinterpret_cast<__half2*>(base8 + SM::kRingOffset);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base8 + SM::kBarOffset);
-    float* red = reinterpret_cast<float*>(base8 + SM::kRedOffset);
-    const int tid = threadIdx.x;
-    const int sl = tid / C::T;
-    const int t = tid % C::T;
-    const int sb = sl * C::N;
-    const int ls = log2_pow2(scale);
-    const int64_t ntiles = (batch + C::S - 1) / C::S;
-    dbg_set_err(err);
-
-    RingInFlight inflight;  // thread 0's copies in flight
-    // copy the tile of the block's iteration `j` into slot j mod D (thread 0 only)
-    auto issue = [&](int64_t j) {
-        const int slot = (int)(j % D);
-        const int64_t tile = blockIdx.x + j * gridDim.x;
-        const int64_t first = tile * C::S;
-        const int64_t left = batch - first;
-        const uint32_t bytes = (uint32_t)((left < C::S ? left : C::S) * C::N * 4);
-        mbar_arrive_expect_tx(&bars[slot], bytes);
-        bulk_copy_g2s(ring + slot * TILE, in + first * C::N, bytes, &bars[slot]);
-        inflight.issued(slot, (uint32_t)((j / D) & 1));
-    };
-    if (tid == 0) {
-        for (int d = 0; d < D; ++d) mbar_init(&bars[d], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (tid == 0 && !stall) {
-        for (int d = 0; d < D; ++d)
-            if (blockIdx.x + (int64_t)d * gridDim.x < ntiles) issue(d);
-    }
-    TcCtx tc;  // FP32 butterflies only
-    bool dead = false;
-    if (stall) {  // failure-detection test mode, as in fft_stockham_ring_kernel
-        if (!mbar_wait_bounded(&bars[0], 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
-        dead = true;
-    }
-    int buf = 0;
-    int64_t it = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-        const int slot = (int)(it % D);
-        const uint32_t parity = (uint32_t)((it / D) & 1);
-        const int64_t sig = tile * C::S + sl;
-        const bool in_range = sig < batch;
-        const int ein = in_range ? (int)in_exp[sig] : 0;
-        if (!dead) {
-            if (mbar_wait_bounded(&bars[slot], parity, wait_ns)) {
-                inflight.completed(slot);
-            } else {
-                dead = true;
-                atomicCAS(err, 0, kErrTimeout);
-            }
-        }
-        float2 v[C::E];
-        gather_tile_c32<C, INV>(v, ring + slot * TILE, sb, t);
-        twist_and_dft<C, 0>(v, t, tw, tc);
-        float2* b = smem + buf * TILE;
-        if constexpr (C::kBuffers == 1) __syncthreads();  // previous readers of b are done
-        scatter<C, 0>(v, b, sb, t);
-        __syncthreads();  // every thread is done with ring[slot]
-        if (tid == 0 && !dead && !stall) {
-            if (tile + (int64_t)D * gridDim.x < ntiles) {
-                fence_proxy_async_smem();
-                issue(it + D);
-            }
-        }
-        gather<C, 1>(v, b, sb, t);
-        if constexpr (C::kBuffers == 2) buf ^= 1;
-        twist_and_dft<C, 1>(v, t, tw, tc);
-        rest_stages<C, 2>(v, smem, buf, sb, t, tw, tc);
-        const C32Out o = c32_out_scale(c32_signal_max<C>(v, red), ein, ls);
-        store_last_c32<C, INV>(v, out + sig * C::N, out_exp + sig, t, in_range && !dead, o);
-    }
-    if (tid == 0) inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
 }
 
 // complex32, N = 2..32: one thread owns a whole signal, as in
@@ -1763,7 +1657,7 @@ __global__ void __launch_bounds__(SC::NT)
             float m = 0.0f;
 #pragma unroll
             for (int i = 0; i < N; ++i) m = fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-            const C32Out o = c32_out_scale(m, ein, ls);
+            const C32Out o = c32_out_scale<N>(m, ein, ls);
             const float my = INV ? -o.mult : o.mult;
             float hw[N];  // binary16 pairs as 32-bit words
 #pragma unroll

@@ -2,6 +2,7 @@
 // -DGBFFT_LOG2N=<1..11>.  The build compiles this file once per length, in
 // parallel, and links the objects with the host plan code.
 #include "fft_device.cuh"
+#include "fft_pair.cuh"
 #include "registry.h"
 #include "schedules.h"
 #include "../../include/gbfft.h"
@@ -67,14 +68,46 @@ static KernelEntry c32_entry(int variant) {
     KernelEntry e = generic_entry<C>(variant);
     e.kind = KernelKind::C32;
     e.smem_bytes = C32Smem<C>::kBytes;
-    if constexpr (C::PIPE > 0) {
-        e.kernel_fwd = reinterpret_cast<const void*>(&fft_stockham_c32_ring_kernel<C, false>);
-        e.kernel_inv = reinterpret_cast<const void*>(&fft_stockham_c32_ring_kernel<C, true>);
-    } else {
-        e.kernel_fwd = reinterpret_cast<const void*>(&fft_stockham_c32_kernel<C, false>);
-        e.kernel_inv = reinterpret_cast<const void*>(&fft_stockham_c32_kernel<C, true>);
-    }
+    e.kernel_fwd = reinterpret_cast<const void*>(&fft_stockham_c32_kernel<C, false>);
+    e.kernel_inv = reinterpret_cast<const void*>(&fft_stockham_c32_kernel<C, true>);
     return e;
+}
+
+// two signals per thread (XB = 6)
+template <class C>
+static KernelEntry pair_c32_entry(int variant) {
+    KernelEntry e{};
+    e.log2n = C::LOG2N;
+    e.variant = variant;
+    e.kind = KernelKind::C32;
+    e.elems_per_thread = C::E;
+    e.signals_per_block = C::S;
+    e.threads_per_block = C::NT;
+    e.smem_bytes = C::kSmemBytes;
+    e.num_stages = C::M;
+    for (int s = 0; s < 4; ++s) e.radix[s] = C::radix(s);
+    e.min_blocks = C::MINB;
+    e.pipeline = C::D;
+    e.twiddles = C::kTwiddles;
+    if constexpr (C::kWarpLocal) {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_pair_c32_warp_kernel<C, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_pair_c32_warp_kernel<C, true>);
+    } else {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_pair_c32_ring_kernel<C, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_pair_c32_ring_kernel<C, true>);
+    }
+    e.fill_twiddles = &fill_generic_twiddles<C>;
+    return e;
+}
+
+template <int L, int E, int S, int R0, int R1, int R2, int R3, int MINB, int PIPE, int XB>
+static KernelEntry c32_row(int variant) {
+    if constexpr (XB == 6) {
+        return pair_c32_entry<PairCfg<L, E, S, R0, R1, R2, R3, MINB, PIPE>>(variant);
+    } else {
+        static_assert(PIPE == 0, "one signal per thread group: direct loads");
+        return c32_entry<Cfg<L, E, S, R0, R1, R2, R3, MINB, 0, 0, XB, 0>>(variant);
+    }
 }
 
 template <class SC>
@@ -202,7 +235,7 @@ int GBFFT_ENTRIES_FN(GBFFT_LOG2N)(gbfft::KernelEntry* out, int max) {
     GBFFT_SMALL_SCHEDULES(GBFFT_SX)
 #undef GBFFT_SX
 #define GBFFT_CX(L, V, E, S, R0, R1, R2, R3, MINB, PIPE, XB) \
-    GBFFT_ONLY_##L(put(c32_entry<Cfg<L, E, S, R0, R1, R2, R3, MINB, PIPE, 0, XB, 0>>(V));)
+    GBFFT_ONLY_##L(put(c32_row<L, E, S, R0, R1, R2, R3, MINB, PIPE, XB>(V));)
     GBFFT_C32_SCHEDULES(GBFFT_CX)
 #undef GBFFT_CX
 #define GBFFT_SCX(L, V, W, U, CH) GBFFT_ONLY_##L(put(small_c32_entry<SmallC32Cfg<L, W, U, CH>>(V));)

@@ -118,26 +118,36 @@
     SX(5, 2, 4, 1, 0)
 
 // complex32-storage rows (FFT_C32): CX(log2N, variant, E, S, R0..R3, MINB,
-// PIPE, XB) as in GX, the Stockham kernel with binary16 loads/stores and
-// per-signal exponents, FP32 arithmetic; PIPE >= 2 stages the binary16 tiles
-// through a bulk-copy ring.  A length's first complex32 row is its default;
-// for N <= 32 that is the one-thread-per-signal SCX row further down.
+// PIPE, XB).  XB = 6 (N >= 64): two signals per thread, packed FP32 arithmetic
+// (fft_pair.cuh), S / 2 signal pairs and S N / (2 E) threads per block, a ring
+// of PIPE bulk-copied tiles per warp (N <= 512) or per block.  XB = 0: the
+// Stockham kernel with binary16 loads/stores, one signal per thread group.
+// A length's first complex32 row is its default; for N <= 32 that is the
+// one-thread-per-signal SCX row further down.
+//
+// Why the defaults are shaped so (2^27 elements, device time, against the
+// one-signal-per-thread kernels they replaced, whose stored values and
+// exponents they reproduce bit for bit): N = 64 244 -> 169 us, 128 241 -> 178,
+// 256 210 -> 180, 512 285 -> 208, 1024 303 -> 220, 2048 302 -> 239.  Blocks of
+// 64 threads at N = 1024 (128: 237 us), because its barriers then join two
+// warps only; one ring slot, because a second one costs the fourth block per SM
+// (N = 1024 and 2048: 252 and 262 us with two slots and three blocks).
 #define GBFFT_C32_SCHEDULES(CX)                   \
     CX(1, 3, 2, 256, 2, 0, 0, 0, 1, 0, 0)        \
     CX(2, 5, 2, 128, 2, 2, 0, 0, 1, 0, 0)        \
     CX(3, 4, 4, 128, 2, 4, 0, 0, 1, 0, 0)        \
     CX(4, 4, 8, 128, 4, 4, 0, 0, 1, 0, 0)        \
     CX(5, 4, 16, 128, 8, 4, 0, 0, 1, 0, 0)       \
-    CX(6, 1, 16, 64, 8, 8, 0, 0, 1, 0, 0)        \
-    CX(7, 5, 16, 32, 8, 16, 0, 0, 1, 0, 0)       \
-    CX(8, 18, 16, 16, 16, 16, 0, 0, 3, 2, 1)      \
-    CX(8, 6, 16, 16, 16, 16, 0, 0, 1, 0, 0)      \
-    CX(9, 2, 16, 8, 8, 8, 8, 0, 2, 0, 0)         \
-    CX(10, 8, 16, 2, 8, 16, 8, 0, 2, 3, 0)       \
-    CX(10, 9, 16, 2, 8, 16, 8, 0, 2, 0, 0)       \
-    CX(11, 8, 16, 1, 8, 16, 16, 0, 3, 3, 0)      \
-    CX(11, 9, 16, 1, 8, 16, 16, 0, 3, 0, 0)      \
-    CX(8, 5, 16, 8, 16, 16, 0, 0, 5, 2, 1)
+    CX(6, 1, 16, 64, 8, 8, 0, 0, 4, 1, 6)        \
+    CX(7, 5, 16, 32, 8, 16, 0, 0, 4, 1, 6)       \
+    CX(8, 18, 16, 8, 16, 16, 0, 0, 8, 1, 6)      \
+    CX(8, 6, 16, 16, 16, 16, 0, 0, 3, 2, 6)      \
+    CX(9, 2, 16, 8, 8, 8, 8, 0, 4, 1, 6)         \
+    CX(10, 8, 16, 2, 8, 16, 8, 0, 8, 1, 6)       \
+    CX(10, 9, 16, 4, 8, 16, 8, 0, 4, 1, 6)       \
+    CX(11, 8, 16, 2, 8, 16, 16, 0, 4, 1, 6)      \
+    CX(11, 9, 16, 2, 8, 16, 16, 0, 3, 2, 6)      \
+    CX(8, 5, 16, 16, 16, 16, 0, 0, 4, 1, 6)
 
 // complex32 one-thread-per-signal rows (N <= 32): SCX(log2N, variant, warps
 // per block, 32-signal groups per warp tile, cache hints)
