@@ -13,6 +13,7 @@ built extension, calls raise.
 from __future__ import annotations
 
 import collections
+import functools
 import threading
 
 import torch
@@ -58,6 +59,23 @@ def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_leas
         raise ValueError(f"{name} has {t.numel()} elements, needs {'at least ' if at_least else ''}{numel}")
 
 
+# The two queries every call needs, without the wrappers' device objects,
+# context managers and stream objects (together about 4 us a call).
+_current_device = torch._C._cuda_getDevice
+_current_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
+def _enqueue(index: int, stream, call, *args) -> None:
+    """call(*args, raw stream) with CUDA device `index` current, on `stream` or
+    that device's current stream."""
+    raw = _current_raw_stream(index) if stream is None else stream.cuda_stream
+    if _current_device() == index:
+        call(*args, raw)
+    else:
+        with torch.cuda.device(index):
+            call(*args, raw)
+
+
 class Plan:
     """One planned transform: length ``n``, ``batch`` signals, a direction.
 
@@ -96,9 +114,7 @@ class Plan:
             out = torch.empty_like(x)
         else:
             _check_buffer(out, "out", torch.complex64, self.device, self.n * self.batch)
-        with torch.cuda.device(x.device):
-            s = stream if stream is not None else torch.cuda.current_stream(x.device)
-            fft_execute(self.handle, x.data_ptr(), out.data_ptr(), s.cuda_stream)
+        _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
     def execute_c32(self, x: torch.Tensor, x_exp: torch.Tensor, out: torch.Tensor | None = None,
@@ -116,10 +132,8 @@ class Plan:
             out_exp = torch.empty(self.batch, dtype=torch.int8, device=x.device)
         else:
             _check_buffer(out_exp, "out_exp", torch.int8, self.device, self.batch)
-        with torch.cuda.device(x.device):
-            s = stream if stream is not None else torch.cuda.current_stream(x.device)
-            fft_execute_c32(self.handle, x.data_ptr(), x_exp.data_ptr(), out.data_ptr(),
-                            out_exp.data_ptr(), s.cuda_stream)
+        _enqueue(self.device.index, stream, fft_execute_c32, self.handle, x.data_ptr(), x_exp.data_ptr(),
+                 out.data_ptr(), out_exp.data_ptr())
         return out, out_exp
 
     def execute_host(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
@@ -191,9 +205,7 @@ class RaggedPlan:
             out = torch.empty_like(x)
         else:
             _check_buffer(out, "out", torch.complex64, self.device, self.total, at_least=True)
-        with torch.cuda.device(x.device):
-            s = stream if stream is not None else torch.cuda.current_stream(x.device)
-            fft_execute(self.handle, x.data_ptr(), out.data_ptr(), s.cuda_stream)
+        _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
     def capture(self, x: torch.Tensor, out: torch.Tensor) -> "torch.cuda.CUDAGraph":
@@ -236,6 +248,9 @@ _cache: "collections.OrderedDict" = collections.OrderedDict()
 _cache_lock = threading.Lock()
 
 
+_device_name = functools.lru_cache(maxsize=64)(str)
+
+
 def _retire(p: Plan) -> None:
     """Destroy an evicted plan once no kernel of it can still be running."""
     torch.cuda.synchronize(p.device)
@@ -244,7 +259,7 @@ def _retire(p: Plan) -> None:
 
 def get_plan(n: int, batch: int, inverse: bool, normalized: bool, device, dtype: str = "c64",
              scale_forward: bool = False) -> Plan:
-    key = (str(device), n, batch, inverse, normalized, dtype, scale_forward)
+    key = (_device_name(device), n, batch, inverse, normalized, dtype, scale_forward)
     with _cache_lock:
         p = _cache.get(key)
         if p is not None:
@@ -276,7 +291,9 @@ def _run(x: torch.Tensor, inverse: bool, normalized: bool = True, dtype: str = "
     x = x.contiguous()
     batch = x.numel() // n if n > 0 else 0
     plan = get_plan(n, batch, inverse, normalized, x.device, dtype, scale_forward)
-    return plan.execute(x)
+    out = torch.empty_like(x)
+    _enqueue(plan.device.index, None, fft_execute, plan.handle, x.data_ptr(), out.data_ptr())
+    return out
 
 
 def fft(x: torch.Tensor, dtype: str = "c64") -> torch.Tensor:
