@@ -258,7 +258,9 @@ GBFFT_API fft_status_t fft_plan_get_info(fft_plan_t plan, fft_plan_info_t* info)
  * work-group factor, Sec. 4).  fft_variant_count returns how many (0 for an
  * invalid length); fft_set_default_variant chooses the FP32 one later plans of
  * that length use (process-wide; the autotuner calls it); plans already made
- * keep theirs.  fft_get_default_variant returns the current choice or -1.
+ * keep theirs.  fft_get_default_variant returns the current choice or -1; the
+ * initial choice, 0, lets a plan take the compiled schedule for its n * batch
+ * (fft_plan_get_info reports which).
  */
 GBFFT_API int fft_variant_count(int64_t n);
 GBFFT_API fft_status_t fft_set_default_variant(int64_t n, int variant);

@@ -520,8 +520,8 @@ struct Cfg {
     static_assert(!kPadSlot || (TC_ == 0 && (N + T) % 2 == 0),
                   "padded slots: FP32, every signal on a 16-byte boundary");
     // a signal spanning warps finds its maximum through shared memory after a
-    // block barrier, so its first stage cannot be a tensor-core one
-    static_assert(!kTcSignalScale || (R0 != 16 && PIPE >= 2 && NT <= 256),
+    // block barrier, so its first stage cannot run on the tensor cores
+    static_assert(!kTcSignalScale || ((R0 != 16 || kTcLastOnly) && PIPE >= 2 && NT <= 256),
                   "FP16 per-signal scale: signals spanning warps only in ring kernels");
     static_assert(TC == 0 || (E == 16 && NT % 128 == 0 && (kTcCols == 32 || kTcCols == 64 || kTcCols == 128)),
                   "tensor-core radix-16 stages need one 16-point butterfly per thread and 128-row tiles");

@@ -36,7 +36,7 @@ using gbfft::KernelKind;
 struct LengthVariants {
     KernelEntry v[GBFFT_MAX_VARIANTS];
     int count = 0;
-    std::atomic<int> preferred{0};  // variant new plans use unless told otherwise
+    std::atomic<int> preferred{0};  // FP32 variant new plans use unless told otherwise; 0: by size
 };
 
 LengthVariants* registry() {
@@ -56,6 +56,30 @@ LengthVariants* registry() {
         table[11].count = gbfft_entries_11(table[11].v, GBFFT_MAX_VARIANTS);
     });
     return table;
+}
+
+// The variant of a plan that names none: type `tc` (0 FP32, 1 FP16 / 2 BF16
+// tensor cores), calls of `elems` elements.
+int default_variant(int log2n, int tc, int64_t elems) {
+    struct Row {
+        int log2n, tc;
+        int64_t max_elems;
+        int variant;
+    };
+#define GBFFT_DX(L, TC, MAX, V) {L, TC, MAX, V},
+    static constexpr Row kRows[] = {GBFFT_SIZE_DEFAULTS(GBFFT_DX)};
+#undef GBFFT_DX
+    const LengthVariants& lv = registry()[log2n];
+    int fallback = 0;
+    if (tc != 0) {
+        while (fallback < lv.count && lv.v[fallback].tc != tc) ++fallback;
+        if (fallback == lv.count) return default_variant(log2n, 0, elems);  // no radix-16 stage: FP32
+    } else if (const int preferred = lv.preferred.load()) {
+        return preferred;
+    }
+    for (const Row& r : kRows)
+        if (r.log2n == log2n && r.tc == tc && elems <= r.max_elems) return r.variant;
+    return fallback;
 }
 
 int ilog2(int64_t n) {
@@ -129,11 +153,11 @@ cudaError_t plan_malloc(void** ptr, size_t bytes) {
 }
 
 // Registry lookup for other host translation units: the kernel entry of
-// `variant` (or of the length's current default when variant < 0), or NULL.
-const KernelEntry* lookup_entry(int log2n, int variant) {
+// `variant` (or of the FP32 default for `elems` elements when variant < 0), or NULL.
+const KernelEntry* lookup_entry(int log2n, int variant, int64_t elems) {
     if (log2n < GBFFT_MIN_LOG2N || log2n > GBFFT_MAX_LOG2N) return nullptr;
     LengthVariants* lv = &registry()[log2n];
-    if (variant < 0) variant = lv->preferred.load();
+    if (variant < 0) variant = default_variant(log2n, 0, elems);
     if (variant >= lv->count || !lv->v[variant].kernel_fwd) return nullptr;
     return &lv->v[variant];
 }
@@ -342,16 +366,12 @@ fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int direction, int dty
     const bool want_c32 = dtype == FFT_C32;
     int variant = (int)((flags & FFT_FLAG_VARIANT_MASK) >> 8) - 1;
     if (variant < 0) {
-        // FP32: the length's default.  Tensor-core types: the first variant of
-        // that type; lengths without a radix-16 tensor-core schedule run FP32.
-        // complex32 storage: the first complex32 variant.
-        variant = lv->preferred.load();
-        for (int v = 0; v < lv->count && (want_tc || want_c32); ++v) {
-            const KernelEntry& c = lv->v[v];
-            if (c.kernel_fwd && ((want_c32 && c.kind == KernelKind::C32) || (want_tc && c.tc == want_tc))) {
-                variant = v;
-                break;
-            }
+        // complex32 storage: the first complex32 variant.  Otherwise by size;
+        // lengths without a tensor-core schedule run FP32.
+        if (want_c32) {
+            for (variant = 0; lv->v[variant].kind != KernelKind::C32;) ++variant;  // every length has one
+        } else {
+            variant = default_variant(log2n, want_tc, n * batch);
         }
     }
     if (variant >= lv->count || !lv->v[variant].kernel_fwd) return FFT_ERR_INVALID_VALUE;

@@ -52,9 +52,9 @@ constexpr int64_t kPdlMinElems = int64_t(1) << 22;
 cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, void** args, size_t smem,
                           cudaStream_t stream, int64_t elems);
 
-// Registry lookup (host): the entry of `variant`, or of the length's current
-// default when variant < 0; NULL when there is none.
-const KernelEntry* lookup_entry(int log2n, int variant);
+// Registry lookup (host): the entry of `variant`, or when variant < 0 of the
+// FP32 default for calls of `elems` elements; NULL when there is none.
+const KernelEntry* lookup_entry(int log2n, int variant, int64_t elems);
 
 // Ragged (mixed-length) plans, implemented in fft_ragged.cu.
 struct RaggedState;

@@ -67,7 +67,7 @@
     GX(8, 0, 16, 16, 16, 16, 0, 0, 2, 2, 0, -1, 2) \
     GX(9, 0, 16, 8, 8, 8, 8, 0, 2, 0, 0, 0, 3) \
     GX(9, 1, 16, 8, 8, 8, 8, 0, 1, 0, 0, 0, 0) \
-    GX(10, 0, 16, 2, 8, 16, 8, 0, 2, 2, 0, 0, 2) \
+    GX(10, 0, 16, 1, 16, 4, 16, 0, 6, 2, 0, -1, 2) \
     GX(10, 1, 16, 2, 8, 16, 8, 0, 1, 0, 0, 0, 0) \
     GX(10, 2, 16, 2, 8, 16, 8, 0, 4, 0, 0, 0, 0) \
     GX(10, 3, 16, 2, 8, 16, 8, 0, 2, 3, 0, 0, 0) \
@@ -80,7 +80,7 @@
     GX(10, 12, 16, 2, 8, 16, 8, 0, 5, 2, 2, -2, 0) \
     GX(10, 13, 16, 2, 8, 16, 8, 0, 4, 2, 1, 1, 0) \
     GX(10, 14, 16, 2, 8, 16, 8, 0, 4, 2, 2, 1, 0) \
-    GX(11, 0, 16, 1, 8, 16, 16, 0, 4, 2, 0, -1, 2) \
+    GX(11, 0, 16, 1, 16, 8, 16, 0, 3, 2, 0, -1, 2) \
     GX(11, 1, 16, 1, 8, 16, 16, 0, 1, 0, 0, 0, 0) \
     GX(11, 2, 16, 1, 8, 16, 16, 0, 2, 3, 0, 0, 0) \
     GX(11, 3, 16, 2, 8, 16, 16, 0, 1, 2, 0, 0, 0) \
@@ -99,23 +99,42 @@
     GX(11, 18, 16, 1, 8, 16, 16, 0, 5, 2, 6, -3, 2) \
     GX(11, 19, 16, 1, 8, 16, 16, 0, 5, 2, 0, -1, 2) \
     GX(6, 4, 16, 64, 8, 8, 0, 0, 1, 0, 0, 0, 0) \
-    GX(7, 6, 16, 32, 8, 16, 0, 0, 1, 0, 0, 0, 2)
+    GX(7, 6, 16, 32, 8, 16, 0, 0, 1, 0, 0, 0, 2) \
+    GX(6, 5, 16, 16, 8, 8, 0, 0, 8, 2, 0, -5, 2) \
+    GX(6, 6, 8, 8, 8, 8, 0, 0, 8, 0, 0, 3, 0) \
+    GX(7, 7, 16, 8, 8, 16, 0, 0, 8, 2, 0, -5, 2) \
+    GX(7, 8, 16, 8, 8, 16, 0, 0, 8, 0, 0, 0, 0) \
+    GX(7, 9, 16, 16, 8, 16, 0, 0, 4, 2, 1, -3, 2) \
+    GX(7, 10, 16, 16, 8, 16, 0, 0, 4, 2, 2, -3, 2) \
+    GX(8, 19, 16, 4, 16, 16, 0, 0, 8, 0, 0, 0, 0) \
+    GX(8, 20, 16, 16, 16, 16, 0, 0, 2, 2, 5, -1, 2) \
+    GX(8, 21, 16, 8, 16, 16, 0, 0, 3, 2, 5, -3, 2) \
+    GX(8, 22, 16, 8, 16, 16, 0, 0, 3, 2, 2, -3, 2) \
+    GX(9, 3, 16, 2, 16, 2, 16, 0, 8, 0, 0, 0, 0) \
+    GX(9, 4, 16, 4, 16, 2, 16, 0, 3, 2, 0, -1, 2) \
+    GX(10, 15, 16, 1, 16, 4, 16, 0, 6, 0, 0, 0, 0)
 
 #define GBFFT_SMALL_SCHEDULES(SX) \
     SX(1, 0, 8, 1, 3)                \
     SX(1, 1, 8, 2, 0)                \
+    SX(1, 4, 4, 2, 0)                \
     SX(2, 0, 4, 8, 2)                \
     SX(2, 1, 8, 1, 0)                \
     SX(2, 2, 8, 4, 2)                \
     SX(2, 3, 16, 2, 2)               \
+    SX(2, 6, 2, 2, 0)                \
     SX(3, 0, 8, 4, 0)                \
     SX(3, 1, 8, 1, 0)                \
     SX(3, 2, 4, 4, 0)                \
+    SX(3, 5, 4, 1, 0)                \
     SX(4, 0, 4, 2, 2)                \
     SX(4, 1, 8, 1, 0)                \
     SX(4, 2, 8, 2, 0)                \
+    SX(4, 5, 2, 1, 0)                \
+    SX(4, 6, 2, 2, 0)                \
     SX(5, 0, 2, 2, 0)                \
-    SX(5, 2, 4, 1, 0)
+    SX(5, 2, 4, 1, 0)                \
+    SX(5, 5, 1, 1, 0)
 
 // complex32-storage rows (FFT_C32): CX(log2N, variant, E, S, R0..R3, MINB,
 // PIPE, XB).  XB = 6 (N >= 64): two signals per thread, packed FP32 arithmetic
@@ -157,6 +176,66 @@
     SCX(3, 3, 8, 4, 0)                  \
     SCX(4, 3, 4, 4, 0)                  \
     SCX(5, 3, 4, 2, 0)
+
+// Which row a plan that names none runs, by length, type and size of the call:
+// DX(log2N, tc type, largest n * batch, variant), the first row that fits; past
+// the last one, variant 0 (FP32) or the first variant of the type.  A default
+// set by fft_set_default_variant (the autotuner's) goes before all of this.
+//
+// Calls of up to some 12 M elements are over in a few tiles per SM: small
+// blocks and tiles spread them over more blocks, start their first store sooner
+// and leave a shorter tail, and evict-first direct loads and stores win while
+// the output still fits in L2.  Larger calls want the larger tiles of variant 0
+// (16 KB and more of consecutive bytes per copy).  Device time per call in a
+// captured graph over three rotating buffer pairs, variant 0 (as it was before
+// these rows) against the row, us:
+//   N = 2     2^21.4 9.5 / 6.6     2^23.2 26.3 / 26.2   2^24.3 53.7 / 56.0
+//   N = 4     2^21.4 8.9 / 6.8     2^23.2 28.1 / 25.6   2^24.3 53.5 / 55.8
+//   N = 8     2^16.2 3.8 / 1.6     2^22.2 17.1 / 13.0   (row 2) 2^23.6 34.1 / 32.9
+//   N = 16    2^22.2 15.8 / 13.7   2^23.2 27.1 / 25.9   (row 6) 2^24.7 68.6 / 66.3
+//   N = 32    2^20.6 5.3 / 4.5     2^22.2 14.3 / 13.0   2^24.3 53.0 / 56.4
+//   N = 64    (row 6) 2^20.6 6.4 / 4.2, 2^22.2 14.7 / 12.9   (row 5) 2^23.2 26.4 / 24.8
+//   N = 128   2^20.6 5.9 / 4.7     2^22.2 14.8 / 13.8   2^24.3 51.4 / 53.6
+//   N = 256   2^20.6 5.4 / 4.4     2^22.2 15.0 / 13.7   2^24.3 52.6 / 53.5
+//   N = 512   2^20.6 6.4 / 5.0     2^23.2 28.5 / 26.1   (row 4) 2^25.2 97.7 / 94.8, 2^28 632 / 635
+//   N = 1024  2^21.4 11.0 / 9.0    2^22.5 18.2 / 18.5
+//   N = 2048  2^21.4 11.1 / 9.8    2^21.8 13.3 / 13.5
+// The up-to-2^16 and 2^17 rows of N = 64 and 128 keep those plans on bulk-copy
+// kernels (0.3-0.8 us over the direct rows, 0.4 under variant 0).
+// Tensor-core types, rows of the same arithmetic only: FP16 N = 256 2^22.3
+// 16.1 / 14.9 (row 21), 2^28 672 / 630 (row 20); BF16 N = 256 2^24 43.7 / 41.8
+// (row 22); N = 128 2^28 672 / 638 and 655 / 643.  (Other radix orders were
+// faster still, N = 1024 and 2048 with radix 16 first and last by 2-9%, but
+// they round the operands of other stages to 16 bits.)
+#define GBFFT_SIZE_DEFAULTS(DX) \
+    DX(1, 0, 8 << 20, 4)        \
+    DX(2, 0, 12 << 20, 6)       \
+    DX(3, 0, 8 << 20, 5)        \
+    DX(3, 0, 12 << 20, 2)       \
+    DX(4, 0, 12 << 20, 5)       \
+    DX(4, 0, 30 << 20, 6)       \
+    DX(5, 0, 12 << 20, 5)       \
+    DX(6, 0, 1 << 16, 5)        \
+    DX(6, 0, 6 << 20, 6)        \
+    DX(6, 0, 16 << 20, 5)       \
+    DX(7, 0, 1 << 17, 7)        \
+    DX(7, 0, 12 << 20, 8)       \
+    DX(8, 0, 16 << 20, 19)      \
+    DX(9, 0, 20 << 20, 3)       \
+    DX(9, 0, 160 << 20, 4)      \
+    DX(10, 0, 1 << 20, 0)       \
+    DX(10, 0, 5 << 20, 15)      \
+    DX(11, 0, 3 << 19, 0)       \
+    DX(11, 0, 3 << 20, 1)       \
+    DX(7, 1, 2 << 20, 1)        \
+    DX(7, 1, INT64_MAX, 9)      \
+    DX(7, 2, 2 << 20, 2)        \
+    DX(7, 2, INT64_MAX, 10)     \
+    DX(8, 1, 2 << 20, 1)        \
+    DX(8, 1, 24 << 20, 21)      \
+    DX(8, 1, INT64_MAX, 20)     \
+    DX(8, 2, 1 << 19, 2)        \
+    DX(8, 2, 24 << 20, 22)
 
 #define GBFFT_MIN_LOG2N 1
 #define GBFFT_MAX_LOG2N 11
