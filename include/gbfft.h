@@ -190,15 +190,16 @@ GBFFT_API fft_status_t fft_execute_c32(fft_plan_t plan, const void* in, const in
 /*
  * The planned transform on HOST buffers: batch*n complex64 read from
  * `in_host`, results written to `out_host` (equal, or not overlapping).  The
- * plan must have been made with FFT_FLAG_HOST_STAGING.  Work is split into
+ * plan must have been made with FFT_FLAG_HOST_STAGING.  Page-locked buffers
+ * (cudaHostAlloc / cudaHostRegister, 16-byte aligned) are read and written in
+ * place over the link by one launch on `stream`.  Otherwise work is split into
  * chunks of whole signals; each chunk is copied to one of the plan's device
  * buffers, transformed in place and copied back, the chunks round-robin over
  * the plan's three streams so that host-to-device copies, kernels and
- * device-to-host copies overlap.  Asynchronous with respect to the host: the
- * pipeline starts after work already enqueued on `stream` and `stream` waits
- * for its end (synchronise `stream` before reading out_host).  Host buffers
- * should be page-locked (cudaHostAlloc / cudaHostRegister); pageable memory
- * works but the copies then serialise.  One call at a time per plan.
+ * device-to-host copies overlap (pageable memory works but its copies
+ * serialise); one such call at a time per plan.  Asynchronous with respect to
+ * the host: the work starts after what is already enqueued on `stream`, and
+ * `stream` waits for its end (synchronise `stream` before reading out_host).
  * Errors: FFT_ERR_INVALID_VALUE (no staging, NULL, ragged plan, wrong device),
  * FFT_ERR_OVERLAP, FFT_ERR_CUDA.
  */

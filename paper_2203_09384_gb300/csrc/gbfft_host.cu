@@ -1,6 +1,7 @@
 // Host side of the C-ABI: argument validation, plan construction (radix
 // schedule lookup, FP64 twiddle generation rounded to FP32, launch shape),
 // asynchronous execution and error reporting.  See include/gbfft.h.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <math.h>
@@ -191,11 +192,12 @@ struct gbfft_plan {
 namespace {
 
 // One launch of the plan's kernel over `batch` signals (any batch up to the
-// plan's), grid sized for that batch.
-fft_status_t launch_plain(gbfft_plan* p, const float2* in2, float2* out2, int64_t batch, cudaStream_t stream) {
+// plan's), grid sized for that batch and for `blocks` at most.
+fft_status_t launch_plain(gbfft_plan* p, const float2* in2, float2* out2, int64_t batch, cudaStream_t stream,
+                          int64_t blocks) {
     const KernelEntry* e = p->entry;
     const int64_t tiles = (batch + e->signals_per_block - 1) / e->signals_per_block;
-    const int64_t grid = tiles < p->resident ? tiles : p->resident;
+    const int64_t grid = tiles < blocks ? tiles : blocks;
     const float2* tw = (const float2*)p->d_twiddles;
     float scale = p->scale;
     int* err = p->d_error;
@@ -216,6 +218,56 @@ fft_status_t launch_plain(gbfft_plan* p, const float2* in2, float2* out2, int64_
         return FFT_ERR_CUDA;
     }
     return FFT_OK;
+}
+
+// The device address of `bytes` bytes of page-locked, mapped host memory at
+// `host`, or NULL when that range is anything else (pageable, managed, or
+// reaching beyond one page-locked allocation).
+void* mapped_host_range(const void* host, size_t bytes) {
+    using GetAttribute = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+    static const GetAttribute get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<GetAttribute>(fn);
+    }();
+    cudaPointerAttributes attr;
+    if (!get || cudaPointerGetAttributes(&attr, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (attr.type != cudaMemoryTypeHost || !attr.devicePointer) return nullptr;
+    const CUdeviceptr at = (CUdeviceptr)attr.devicePointer;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    if (get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+        get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS)
+        return nullptr;
+    if (at < start || bytes > size || at - start > size - bytes) return nullptr;
+    return attr.devicePointer;
+}
+
+// Blocks of a transform that reads and writes host memory over the link.  The
+// link moves about 200 GB/s a way, so 1.25 MiB of tiles in flight cover its
+// latency, and more lets the reads of a short call run ahead of the writes that
+// should share the time; long calls take up to 4.75 MiB, where every kernel
+// reaches its best.  2^20 elements of N = 1024: 65 us with 76 blocks, 77 with
+// 304, 89 with all that are resident; 2^24: 807, 813 and 850 us; 2^24 of
+// N = 16: 848, 840 and 881 us.
+int64_t host_blocks(const gbfft_plan* p) {
+    const KernelEntry* e = p->entry;
+    const int64_t per_block = (int64_t)e->signals_per_block * p->n * 8 * (e->pipeline > 1 ? e->pipeline : 1);
+    const int64_t least = int64_t(5) << 18, most = int64_t(19) << 18;
+    int64_t in_flight = p->n * p->batch / 2;  // a sixteenth of the input
+    in_flight = in_flight < least ? least : in_flight > most ? most : in_flight;
+    int64_t blocks = in_flight / per_block;
+    if (blocks < p->sm_count / 4) blocks = p->sm_count / 4;
+    return blocks < p->resident ? blocks : p->resident;
 }
 
 void release_staging(gbfft_plan* p) {
@@ -565,7 +617,7 @@ fft_status_t fft_execute(fft_plan_t p, const void* in, void* out, void* stream) 
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) return FFT_ERR_INVALID_VALUE;
 
-    return launch_plain(p, (const float2*)in, (float2*)out, p->batch, (cudaStream_t)stream);
+    return launch_plain(p, (const float2*)in, (float2*)out, p->batch, (cudaStream_t)stream, p->resident);
 }
 
 fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host, void* stream) {
@@ -579,6 +631,15 @@ fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host,
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) return FFT_ERR_INVALID_VALUE;
     cudaStream_t user = (cudaStream_t)stream;
+    // Page-locked buffers: one launch reads and writes them in place over the
+    // link.  Against the staging copies below (2^16, 2^20, 2^24, 2^26 elements
+    // of N = 1024): 32 -> 16, 109 -> 65, 1116 -> 813, 3534 -> 3182 us, where
+    // the link alone takes 3, 49, 783 and 3130 us with both directions busy.
+    if (((a | b) & 15) == 0) {
+        void* din = mapped_host_range(in_host, bytes);
+        void* dout = a == b ? din : din ? mapped_host_range(out_host, bytes) : nullptr;
+        if (din && dout) return launch_plain(p, (const float2*)din, (float2*)dout, p->batch, user, host_blocks(p));
+    }
     // the pipeline starts after the caller's earlier work ...
     if (cudaEventRecord(p->stage_start, user) != cudaSuccess) goto cuda_fail;
     for (int i = 0; i < p->stages; ++i)
@@ -598,7 +659,7 @@ fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host,
             // order; the three streams overlap both copy directions and kernels
             if (cudaMemcpyAsync(buf, src + first * sig_bytes, nbytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
                 goto cuda_fail;
-            fft_status_t st = launch_plain(p, buf, buf, nsig, s);
+            fft_status_t st = launch_plain(p, buf, buf, nsig, s, p->resident);
             if (st != FFT_OK) return st;
             if (cudaMemcpyAsync(dst + first * sig_bytes, buf, nbytes, cudaMemcpyDeviceToHost, s) != cudaSuccess)
                 goto cuda_fail;
