@@ -314,6 +314,35 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Cluster launch control: take the place of a block of this grid that has not
+// started yet.  The 16-byte answer arrives at `resp` and completes on `bar`.
+__device__ __forceinline__ void steal_request(void* resp, uint64_t* bar) {
+    mbar_arrive_expect_tx(bar, 16);
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+            smem_u32(resp)),
+        "r"(smem_u32(bar))
+        : "memory");
+}
+// The answer once it has arrived: the index of the block whose place was
+// taken, or -1 when every block has started (no further request then).
+__device__ __forceinline__ int64_t steal_answer(const void* resp) {
+    uint32_t ok, x;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, _, _, _}, r;\n\t}"
+        : "=r"(ok), "=r"(x)
+        : "r"(smem_u32(resp))
+        : "memory");
+    return ok ? (int64_t)x : -1;
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -412,13 +441,53 @@ struct RingInFlight {
     }
 };
 
+// The tiles a block works through when tiles are taken from blocks that have
+// not started: its own first, then whatever the requests bring.  One thread
+// asks; at most one request is out at a time, made a whole tile ahead.
+// Handing tiles out in the order blocks become free keeps the tiles in flight
+// close together in HBM, where a fixed stride lets blocks drift apart: at 2^28
+// elements N = 256 646 -> 606 us, N = 512 639 -> 606, N = 2048 645 -> 622.
+struct TileTaker {
+    unsigned char* resp = nullptr;  // 16 bytes, 16-byte aligned
+    uint64_t* bar = nullptr;
+    uint32_t parity = 0;
+    bool out = false;  // a request is under way
+    __device__ __forceinline__ void request() {
+        steal_request(resp, bar);
+        out = true;
+    }
+    // The next tile, or -1 for none; `late` when no answer came in time.
+    __device__ __forceinline__ int64_t take(uint64_t limit_ns, bool& late) {
+        if (!out) return -1;
+        if (!mbar_wait_bounded(bar, parity, limit_ns)) {
+            late = true;
+            return -1;
+        }
+        out = false;
+        parity ^= 1;
+        const int64_t tile = steal_answer(resp);
+        fence_proxy_async_smem();  // the answer has been read before the next one may overwrite it
+        return tile;
+    }
+    // After a wait gave up: take the remaining tiles without working on them
+    // (new blocks would each wait in turn), and leave no answer under way.
+    __device__ __forceinline__ void drain(uint64_t limit_ns) {
+        bool late = false;
+        while (out && !late)
+            if (take(limit_ns, late) >= 0) request();
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Compile-time schedule
 // ---------------------------------------------------------------------------
 template <int LOG2N_, int E_, int S_, int R0, int R1, int R2, int R3, int MINB_ = 1, int PIPE_ = 0, int TC_ = 0,
           int XB_ = 0, int CH_ = 0>
 struct Cfg {
-    static constexpr int CH = CH_;  // cache hints of the HBM loads / stores
+    static constexpr int CH = CH_ & 3;  // cache hints of the HBM loads / stores
+    // CH bit 2 (in-ring schedules): one block per tile is launched, and a
+    // running block takes the tiles of blocks that have not started yet
+    static constexpr bool kSteal = (CH_ & 4) != 0;
     static constexpr int LOG2N = LOG2N_;
     static constexpr int N = 1 << LOG2N_;
     static constexpr int E = E_;          // complex elements per thread
@@ -479,12 +548,17 @@ struct Cfg {
     // scales each butterfly row before its conversion.  BF16: no scale.
     static constexpr bool kTcSignalScale = TC == 1 && T > 32;
     static constexpr bool kTcRowScale = TC == 1 && T <= 32;
-    static constexpr int kTcOffset = (((kSmemElems + kRingElems) * 8 + 8 * PIPE) + 127) / 128 * 128;
+    // after the ring's mbarriers, for tile stealing: the answer, its mbarrier,
+    // and the tile in each slot (-1: no more tiles)
+    static constexpr int kStealOffset = ((kSmemElems + kRingElems) * 8 + 8 * PIPE + 15) / 16 * 16;
+    static constexpr int kRingBytes =
+        kSteal ? kStealOffset + 16 + 8 + 8 * PIPE : (kSmemElems + kRingElems) * 8 + 8 * PIPE;
+    static constexpr int kTcOffset = (kRingBytes + 127) / 128 * 128;
     // A operand (kTcTiles x 8 KiB, unless it lives in the ring slot), B (2 KiB),
     // the MMA-completion mbarrier and the TMEM address slot
     static constexpr int kTcABytes = (kAInRing || kAInTmem) ? 0 : kTcTiles * 8192;
     static constexpr int kTcBytes = TC ? kTcABytes + 2048 + 128 : 0;
-    static constexpr int kSmemBytes = TC ? kTcOffset + kTcBytes : (kSmemElems + kRingElems) * 8 + 8 * PIPE;
+    static constexpr int kSmemBytes = TC ? kTcOffset + kTcBytes : kRingBytes;
     __host__ __device__ static constexpr int radix(int s) {
         return s == 0 ? R0 : s == 1 ? R1 : s == 2 ? R2 : R3;
     }
@@ -513,6 +587,7 @@ struct Cfg {
     static_assert(32 % T == 0 || T % 32 == 0, "T must tile warps");
     static_assert(PIPE == 0 || PIPE >= 2, "the bulk-copy ring needs at least two slots");
     static_assert(!kInRing || PIPE >= 2, "exchanges in the ring slot need the bulk-copy ring");
+    static_assert(!kSteal || (kInRing && PIPE == 2), "tile stealing: in-ring schedules with two slots");
     static_assert(!kShuffle || (M == 2 && R0 == R1 && E == R0 && T == E && T <= 32 && PIPE == 0 && TC_ == 0),
                   "shuffle exchange: two stages N = R x R, one butterfly of R per thread, R lanes per signal");
     static_assert(!kAInRing || TC == 0 || kTcTiles * 8192 <= S * N * 8, "the A operand must fit in a ring slot");
@@ -1247,7 +1322,9 @@ __device__ __forceinline__ void rest_stages_in_ring(float2 (&v)[C::E], float2* b
 // k.  Slot k is refilled at the first barrier of the next tile, when every
 // thread is done with it, so the ring runs D-1 tiles ahead.  Shared memory is
 // the ring alone (plus the tensor-core B operand), so more blocks fit per SM.
-// Waits are bounded as in fft_stockham_ring_kernel.
+// A block's tiles are blockIdx.x, + gridDim.x, ..., or (kSteal) its own and
+// those it takes from blocks that have not started.  Waits are bounded as in
+// fft_stockham_ring_kernel.
 template <class C, bool INV>
 __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_slot_ring_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw,
@@ -1259,6 +1336,8 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     extern __shared__ __align__(16) float2 smem[];
     float2* ring = smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(ring + D * TILE);
+    unsigned char* steal = reinterpret_cast<unsigned char*>(smem) + C::kStealOffset;
+    volatile int64_t* slot_tile = reinterpret_cast<volatile int64_t*>(steal + 24);  // kSteal
     const int tid = threadIdx.x;
     const int sl = tid / C::T;
     const int t = tid % C::T;
@@ -1267,13 +1346,12 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     dbg_set_err(err);
 
     RingInFlight inflight;  // thread 0's copies in flight
-    // copy the tile of the block's iteration `j` into slot j mod D: thread 0
-    // with one copy, or (padded slots) the lanes of warp 0 with one copy per
-    // signal after lane 0 has set the byte count
+    TileTaker taker;        // thread 0's requests (kSteal)
+    // copy `tile` into `slot`, for the use of that slot with phase parity
+    // `parity`: thread 0 with one copy, or (padded slots) the lanes of warp 0
+    // with one copy per signal after lane 0 has set the byte count
     constexpr int kIssuers = C::kPadSlot ? 32 : 1;
-    auto issue = [&](int64_t j) {
-        const int slot = (int)(j % D);
-        const int64_t tile = blockIdx.x + j * gridDim.x;
+    auto issue = [&](int slot, int64_t tile, uint32_t parity) {
         const int64_t first = tile * C::S;
         const int64_t left = batch - first;
         const int nsig = (int)(left < C::S ? left : C::S);
@@ -1281,29 +1359,60 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         if constexpr (C::kPadSlot) {
             const int lane = threadIdx.x & 31;
             if (lane == 0) {
+                if constexpr (C::kSteal) slot_tile[slot] = tile;
                 mbar_arrive_expect_tx(&bars[slot], bytes);
-                inflight.issued(slot, (uint32_t)((j / D) & 1));
+                inflight.issued(slot, parity);
             }
             __syncwarp();
             for (int q = lane; q < nsig; q += 32)
                 bulk_copy_g2s(ring + slot * TILE + q * (C::N + C::kSlotPad), in + (first + q) * C::N,
                               (uint32_t)(C::N * 8), &bars[slot]);
         } else {
+            if constexpr (C::kSteal) slot_tile[slot] = tile;
             mbar_arrive_expect_tx(&bars[slot], bytes);
             bulk_copy_g2s(ring + slot * TILE, in + first * C::N, bytes, &bars[slot]);
-            inflight.issued(slot, (uint32_t)((j / D) & 1));
+            inflight.issued(slot, parity);
+        }
+    };
+    // kSteal (the issuing threads): fill `slot` with the tile the last request
+    // brought and ask for another, or mark the end
+    auto issue_taken = [&](int slot, uint32_t parity) {
+        int64_t tile = -1;
+        if (tid == 0) {
+            bool late = false;
+            tile = taker.take(wait_ns, late);
+            if (late) atomicCAS(err, 0, kErrTimeout);
+        }
+        if constexpr (C::kPadSlot) tile = __shfl_sync(0xffffffffu, tile, 0);
+        if (tile >= 0) {
+            issue(slot, tile, parity);
+            if (tid == 0) taker.request();
+        } else if (tid == 0) {
+            slot_tile[slot] = -1;
+            mbar_arrive(&bars[slot]);
         }
     };
     if (tid == 0) {
         for (int d = 0; d < D; ++d) mbar_init(&bars[d], 1);
+        if constexpr (C::kSteal) {
+            taker.resp = steal;
+            taker.bar = reinterpret_cast<uint64_t*>(steal + 16);
+            mbar_init(taker.bar, 1);
+        }
         fence_mbar_init();
     }
     __syncthreads();
     // stall != 0 is the failure-detection test mode: nothing is issued, so
     // every wait below runs out, records FFT_ERR_TIMEOUT and the kernel ends
     if (tid < kIssuers && !stall) {
-        for (int d = 0; d < D; ++d)
-            if (blockIdx.x + (int64_t)d * gridDim.x < ntiles) issue(d);
+        issue(0, blockIdx.x, 0);
+        if constexpr (C::kSteal) {
+            if (tid == 0) taker.request();
+            issue_taken(1, 0);
+        } else {
+            for (int d = 1; d < D; ++d)
+                if (blockIdx.x + (int64_t)d * gridDim.x < ntiles) issue(d, blockIdx.x + (int64_t)d * gridDim.x, 0);
+        }
     }
     TcCtx tc;
     if constexpr (C::TC != 0) tc_setup<C>(tc, reinterpret_cast<unsigned char*>(smem) + C::kTcOffset, err, wait_ns);
@@ -1312,9 +1421,10 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     if (stall) {  // wait for a phase nothing will complete: must give up after wait_ns
         if (!mbar_wait_bounded(&bars[0], 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         dead = true;
+        if (C::kSteal && tid == 0) taker.request();  // for the drain below
     }
     int64_t it = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+    for (int64_t tile = blockIdx.x; C::kSteal || tile < ntiles; tile += gridDim.x, ++it) {
         const int slot = (int)(it % D);
         const uint32_t parity = (uint32_t)((it / D) & 1);
         if (!dead) {
@@ -1325,23 +1435,34 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
                 atomicCAS(err, 0, kErrTimeout);
             }
         }
+        if constexpr (C::kSteal) tile = dead ? -1 : slot_tile[slot];
         float2* b = ring + slot * TILE;
         if constexpr (C::kAInRing) tc.a = reinterpret_cast<unsigned char*>(b);
         const int64_t sig = tile * C::S + sl;
         float2 v[C::E];
-        gather_tile<C, INV>(v, b, sl * (C::N + C::kSlotPad), t);
-        tc_norm_begin<C>(v, tc);
-        twist_and_dft<C, 0>(v, t, tw, tc);
+        if (!C::kSteal || tile >= 0) {
+            gather_tile<C, INV>(v, b, sl * (C::N + C::kSlotPad), t);
+            tc_norm_begin<C>(v, tc);
+            twist_and_dft<C, 0>(v, t, tw, tc);
+        }
         // order this thread's generic accesses of the previous tile's slot
         // before the bulk copy that refills it, then one barrier: every thread
         // is done with that slot and has read this tile's stage-0 inputs
         // (padded slots: before the dense exchanges overwrite them)
         fence_proxy_async_smem();
-        __syncthreads();
-        if (tid < kIssuers && it > 0 && !stall) {
-            bool go = !dead;
-            if constexpr (C::kPadSlot) go = __shfl_sync(0xffffffffu, go, 0);  // warp 0 follows lane 0
-            if (go && tile + (int64_t)(D - 1) * gridDim.x < ntiles) issue(it - 1 + D);
+        if constexpr (C::kSteal) {
+            // every thread leaves in the same iteration, also when one gave up
+            if (__syncthreads_or(dead) || tile < 0) break;
+            if (tid < kIssuers && it > 0) issue_taken(slot ^ 1, (uint32_t)(((it + 1) / D) & 1));
+        } else {
+            __syncthreads();
+            if (tid < kIssuers && it > 0 && !stall) {
+                bool go = !dead;
+                if constexpr (C::kPadSlot) go = __shfl_sync(0xffffffffu, go, 0);  // warp 0 follows lane 0
+                const int64_t j = it - 1 + D;  // the iteration the freed slot is next used in
+                if (go && tile + (int64_t)(D - 1) * gridDim.x < ntiles)
+                    issue((int)(j % D), tile + (int64_t)(D - 1) * gridDim.x, (uint32_t)((j / D) & 1));
+            }
         }
         tc_norm_end<C>(v, tc);  // signals spanning warps: maxima published before the barrier
         scatter<C, 0>(v, b, sb, t);
@@ -1353,7 +1474,10 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         const float f = tc_store_factor<C>(v, tc, scale);
         store_last<C, INV>(v, out + sig * C::N, t, active, f);
     }
-    if (tid == 0) inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
+    if (tid == 0) {
+        if constexpr (C::kSteal) taker.drain(wait_ns);
+        inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
+    }
     if constexpr (C::TC != 0) tc_teardown<C>(tc);
 }
 
@@ -1364,65 +1488,107 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
 // ---------------------------------------------------------------------------
 template <int LOG2N, int WARPS, int U = 1, int CH_ = 0>
 struct SmallCfg {
-    static constexpr int CH = CH_;  // cache hints of the HBM loads / stores
+    static constexpr int CH = CH_ & 3;  // cache hints of the HBM loads / stores
+    // CH bit 2: one block per tile is launched, and a running block (one warp)
+    // takes the tiles of blocks that have not started
+    static constexpr bool kSteal = (CH_ & 4) != 0;
+    static_assert(!kSteal || WARPS == 1, "tile stealing: one warp per block");
     static constexpr int N = 1 << LOG2N;
     static constexpr int H = N / 2;  // float4 slots per signal
     static constexpr int WARPS_PER_BLOCK = WARPS;
     static constexpr int UNROLL = U;  // 32-signal groups a warp keeps in flight per iteration
     static constexpr int NT = 32 * WARPS;
-    static constexpr int kSmemBytes = WARPS * 32 * U * H * 16;
+    static constexpr int kSlabBytes = WARPS * 32 * U * H * 16;
+    static constexpr int kSmemBytes = kSlabBytes + (kSteal ? 32 : 0);  // + the answer and its mbarrier
 };
 
 // One warp tile = 32*U consecutive signals (contiguous in HBM): loaded with
 // coalesced 128-bit copies into the warp's shared-memory slab, then each lane
 // transforms U signals of its own, then the slab is stored back the same way.
 template <class SC, bool INV>
+__device__ __forceinline__ void small_tile(const float2* in, float2* out, int64_t batch, float scale, float4* sm,
+                                           int64_t wt) {
+    constexpr int N = SC::N, H = SC::H, U = SC::UNROLL;
+    constexpr int TS = 32 * U;  // signals per warp tile
+    const int lane = threadIdx.x & 31;
+    const int64_t first = wt * TS;
+    const int64_t left = batch - first;
+    const int valid4 = (int)((left < TS ? left : TS) * H);
+    const float4* src = reinterpret_cast<const float4*>(in + first * N);
+    float4* dst = reinterpret_cast<float4*>(out + first * N);
+#pragma unroll
+    for (int i = 0; i < U * H; ++i) {
+        const int p = lane + 32 * i;
+        if (p < valid4) sm[swz16<SC::N>(p)] = ld_stream4v<SC::CH>(src + p);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int sig = u * 32 + lane;
+        float2 v[N];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            float4 f = sm[swz16<SC::N>(sig * H + i)];
+            v[2 * i] = make_float2(f.x, INV ? -f.y : f.y);
+            v[2 * i + 1] = make_float2(f.z, INV ? -f.w : f.w);
+        }
+        Dft<N>::run(v);
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = make_float2(v[i].x * scale, (INV ? -v[i].y : v[i].y) * scale);
+#pragma unroll
+        for (int i = 0; i < H; ++i)
+            sm[swz16<SC::N>(sig * H + i)] = make_float4(v[2 * i].x, v[2 * i].y, v[2 * i + 1].x, v[2 * i + 1].y);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < U * H; ++i) {
+        const int p = lane + 32 * i;
+        if (p < valid4) st_stream4v<SC::CH>(dst + p, sm[swz16<SC::N>(p)]);
+    }
+    __syncwarp();
+}
+
+template <class SC, bool INV>
 __global__ void __launch_bounds__(SC::NT) fft_small_kernel(const float2* in, float2* out, int64_t batch,
                                                            float scale) {
     pdl_enter();
-    constexpr int N = SC::N, H = SC::H, W = SC::WARPS_PER_BLOCK, U = SC::UNROLL;
-    constexpr int TS = 32 * U;  // signals per warp tile
+    constexpr int W = SC::WARPS_PER_BLOCK, TS = 32 * SC::UNROLL;
     extern __shared__ __align__(16) float4 smem4[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float4* sm = smem4 + warp * (TS * H);
+    const int warp = threadIdx.x >> 5;
     const int64_t wtiles = (batch + TS - 1) / TS;
-    for (int64_t wt = (int64_t)blockIdx.x * W + warp; wt < wtiles; wt += (int64_t)gridDim.x * W) {
-        const int64_t first = wt * TS;
-        const int64_t left = batch - first;
-        const int valid4 = (int)((left < TS ? left : TS) * H);
-        const float4* src = reinterpret_cast<const float4*>(in + first * N);
-        float4* dst = reinterpret_cast<float4*>(out + first * N);
-#pragma unroll
-        for (int i = 0; i < U * H; ++i) {
-            const int p = lane + 32 * i;
-            if (p < valid4) sm[swz16<SC::N>(p)] = ld_stream4v<SC::CH>(src + p);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int sig = u * 32 + lane;
-            float2 v[N];
-#pragma unroll
-            for (int i = 0; i < H; ++i) {
-                float4 f = sm[swz16<SC::N>(sig * H + i)];
-                v[2 * i] = make_float2(f.x, INV ? -f.y : f.y);
-                v[2 * i + 1] = make_float2(f.z, INV ? -f.w : f.w);
-            }
-            Dft<N>::run(v);
-#pragma unroll
-            for (int i = 0; i < N; ++i) v[i] = make_float2(v[i].x * scale, (INV ? -v[i].y : v[i].y) * scale);
-#pragma unroll
-            for (int i = 0; i < H; ++i)
-                sm[swz16<SC::N>(sig * H + i)] = make_float4(v[2 * i].x, v[2 * i].y, v[2 * i + 1].x, v[2 * i + 1].y);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < U * H; ++i) {
-            const int p = lane + 32 * i;
-            if (p < valid4) st_stream4v<SC::CH>(dst + p, sm[swz16<SC::N>(p)]);
-        }
-        __syncwarp();
+    for (int64_t wt = (int64_t)blockIdx.x * W + warp; wt < wtiles; wt += (int64_t)gridDim.x * W)
+        small_tile<SC, INV>(in, out, batch, scale, smem4 + warp * (TS * SC::H), wt);
+}
+
+// The same with one warp per block, taking the tiles of unstarted blocks; the
+// request for the next tile runs behind the current one.  (`tw` and `stall` are
+// accepted so that the host launches it like the longer lengths' kernels.)
+template <class SC, bool INV>
+__global__ void __launch_bounds__(SC::NT)
+    fft_small_steal_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw, float scale,
+                           int* err, uint64_t wait_ns, int stall) {
+    pdl_enter();
+    extern __shared__ __align__(16) float4 smem4[];
+    unsigned char* steal = reinterpret_cast<unsigned char*>(smem4) + SC::kSlabBytes;
+    TileTaker taker;  // lane 0's requests
+    if (threadIdx.x == 0) {
+        taker.resp = steal;
+        taker.bar = reinterpret_cast<uint64_t*>(steal + 16);
+        mbar_init(taker.bar, 1);
+        fence_mbar_init();
+        taker.request();
     }
+    for (int64_t tile = blockIdx.x; tile >= 0;) {
+        small_tile<SC, INV>(in, out, batch, scale, smem4, tile);
+        if (threadIdx.x == 0) {
+            bool late = false;
+            tile = taker.take(wait_ns, late);
+            if (late) atomicCAS(err, 0, kErrTimeout);
+            if (tile >= 0) taker.request();
+        }
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+    }
+    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up
 }
 
 // ---------------------------------------------------------------------------

@@ -45,6 +45,7 @@ static KernelEntry generic_entry(int variant) {
     for (int s = 0; s < 4; ++s) e.radix[s] = C::radix(s);
     e.min_blocks = C::MINB;
     e.pipeline = C::PIPE;
+    e.steal = C::kSteal;
     e.tc = C::TC;
     e.tc_stages = C::kTcStages;
     e.tmem_cols = C::TC ? C::kTcCols : 0;
@@ -149,8 +150,14 @@ static KernelEntry small_entry(int variant) {
     e.tc = 0;
     e.tmem_cols = 0;
     e.twiddles = 0;
-    e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_kernel<SC, false>);
-    e.kernel_inv = reinterpret_cast<const void*>(&fft_small_kernel<SC, true>);
+    e.steal = SC::kSteal;
+    if constexpr (SC::kSteal) {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_steal_kernel<SC, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_small_steal_kernel<SC, true>);
+    } else {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_kernel<SC, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_small_kernel<SC, true>);
+    }
     e.fill_twiddles = &fill_nothing;
     return e;
 }

@@ -217,7 +217,7 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
     float scale = scaled ? 1.0f / (float)n : 1.0f;
     const int64_t tiles = (batch + e->signals_per_block - 1) / e->signals_per_block;
     const int64_t resident = (int64_t)d->sm_count * per_sm;
-    const int64_t grid = tiles < resident ? tiles : resident;
+    const int64_t grid = e->steal || tiles < resident ? tiles : resident;
     const float2* in2 = (const float2*)in;
     float2* out2 = (float2*)out;
     const float2* tw = d->scratch;
@@ -225,7 +225,7 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
     uint64_t wait_ns = 4000000000ull;
     const void* kernel = inverse ? e->kernel_inv : e->kernel_fwd;
     cudaError_t ce;
-    if (e->kind == gbfft::KernelKind::Small) {
+    if (e->kind == gbfft::KernelKind::Small && !e->steal) {
         void* args[] = {&in2, &out2, &batch, &scale};
         ce = cudaLaunchKernel(kernel, dim3((unsigned)grid), dim3(e->threads_per_block), args, (size_t)e->smem_bytes,
                               s);

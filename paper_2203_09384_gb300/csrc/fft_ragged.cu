@@ -436,10 +436,6 @@ __device__ __forceinline__ void slot_sync() {
     }
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 template <class C, int s>
 __device__ __forceinline__ void slot_stages(float2 (&v)[C::E], float2* b, int sb, int t, const float2* __restrict__ tw,
                                             TcCtx& tc) {

@@ -60,8 +60,9 @@ LengthVariants* registry() {
 }
 
 // The variant of a plan that names none: type `tc` (0 FP32, 1 FP16 / 2 BF16
-// tensor cores), calls of `elems` elements.
-int default_variant(int log2n, int tc, int64_t elems) {
+// tensor cores), calls of `elems` elements.  Without `steal`, the last row for
+// smaller calls in place of one that needs a block per tile.
+int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
     struct Row {
         int log2n, tc;
         int64_t max_elems;
@@ -74,12 +75,15 @@ int default_variant(int log2n, int tc, int64_t elems) {
     int fallback = 0;
     if (tc != 0) {
         while (fallback < lv.count && lv.v[fallback].tc != tc) ++fallback;
-        if (fallback == lv.count) return default_variant(log2n, 0, elems);  // no radix-16 stage: FP32
+        if (fallback == lv.count) return default_variant(log2n, 0, elems, steal);  // no radix-16 stage: FP32
     } else if (const int preferred = lv.preferred.load()) {
         return preferred;
     }
-    for (const Row& r : kRows)
-        if (r.log2n == log2n && r.tc == tc && elems <= r.max_elems) return r.variant;
+    for (const Row& r : kRows) {
+        if (r.log2n != log2n || r.tc != tc || (!steal && lv.v[r.variant].steal)) continue;
+        if (elems <= r.max_elems) return r.variant;
+        if (!steal) fallback = r.variant;
+    }
     return fallback;
 }
 
@@ -170,14 +174,22 @@ struct gbfft_plan {
     uint32_t flags = 0;
     int device = -1;
     int sm_count = 0;
-    const KernelEntry* entry = nullptr;
-    const void* kernel = nullptr;
-    float* d_twiddles = nullptr;  // interleaved complex64
+    // a kernel, its twiddle table (interleaved complex64) and the blocks of it
+    // that fit on the device at once
+    struct Launch {
+        const KernelEntry* entry = nullptr;
+        const void* kernel = nullptr;
+        const float* d_twiddles = nullptr;
+        int64_t resident = 0;
+    };
+    Launch dev;       // on device buffers
+    Launch host;      // on mapped host buffers (FFT_FLAG_HOST_STAGING)
+    const KernelEntry* entry = nullptr;  // dev.entry
+    void* d_tables = nullptr;            // twiddle tables, then the error word
     int* d_error = nullptr;
     int64_t grid = 0;
     float scale = 1.0f;
     uint64_t wait_ns = kDefaultWaitNs;
-    int64_t resident = 0;                  // blocks that fit on the device at once
     gbfft::RaggedState* ragged = nullptr;  // set for mixed-length plans
     // host-buffer pipeline (FFT_FLAG_HOST_STAGING): device chunk buffers,
     // one stream each, and the events that tie them to the caller's stream
@@ -191,26 +203,27 @@ struct gbfft_plan {
 
 namespace {
 
-// One launch of the plan's kernel over `batch` signals (any batch up to the
-// plan's), grid sized for that batch and for `blocks` at most.
-fft_status_t launch_plain(gbfft_plan* p, const float2* in2, float2* out2, int64_t batch, cudaStream_t stream,
-                          int64_t blocks) {
-    const KernelEntry* e = p->entry;
+// One launch of `l` over `batch` signals (any batch up to the plan's), grid
+// sized for that batch and for `blocks` at most (kernels that take tiles of
+// unstarted blocks need one block per tile).
+fft_status_t launch_plain(gbfft_plan* p, const gbfft_plan::Launch& l, const float2* in2, float2* out2, int64_t batch,
+                          cudaStream_t stream, int64_t blocks) {
+    const KernelEntry* e = l.entry;
     const int64_t tiles = (batch + e->signals_per_block - 1) / e->signals_per_block;
-    const int64_t grid = tiles < blocks ? tiles : blocks;
-    const float2* tw = (const float2*)p->d_twiddles;
+    const int64_t grid = e->steal || tiles < blocks ? tiles : blocks;
+    const float2* tw = (const float2*)l.d_twiddles;
     float scale = p->scale;
     int* err = p->d_error;
     uint64_t wait_ns = p->wait_ns;
     cudaError_t ce;
-    if (e->kind == KernelKind::Small) {
+    if (e->kind == KernelKind::Small && !e->steal) {
         void* args[] = {&in2, &out2, &batch, &scale};
-        ce = gbfft::launch_kernel(p->kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
+        ce = gbfft::launch_kernel(l.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
                                   (size_t)e->smem_bytes, stream, batch * p->n);
     } else {
         int stall = (p->flags & FFT_FLAG_TEST_STALL) ? 1 : 0;
         void* args[] = {&in2, &out2, &batch, &tw, &scale, &err, &wait_ns, &stall};
-        ce = gbfft::launch_kernel(p->kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
+        ce = gbfft::launch_kernel(l.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
                                   (size_t)e->smem_bytes, stream, batch * p->n);
     }
     if (ce != cudaSuccess) {
@@ -218,6 +231,30 @@ fft_status_t launch_plain(gbfft_plan* p, const float2* in2, float2* out2, int64_
         return FFT_ERR_CUDA;
     }
     return FFT_OK;
+}
+
+// Resident blocks of one kernel on device `dev`, after its shared-memory
+// opt-in; 0 with a CUDA error, -1 when it cannot run here.
+int64_t resident_blocks(const KernelEntry* e, const void* kernel, int dev, int sms) {
+    if (e->smem_bytes > 48 * 1024 &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, e->smem_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, e->threads_per_block, e->smem_bytes) !=
+            cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (e->tmem_cols > 0) per_sm = occupancy_without_tmem(kernel, e->threads_per_block, e->smem_bytes, dev);
+    if (e->tmem_cols > 0 && per_sm * e->tmem_cols > 512) {
+        // every resident block holds its TMEM columns for its whole life; more
+        // than 512 per SM would leave a block waiting for columns forever
+        per_sm = 512 / e->tmem_cols;
+    }
+    return per_sm < 1 ? -1 : (int64_t)sms * per_sm;
 }
 
 // The device address of `bytes` bytes of page-locked, mapped host memory at
@@ -260,14 +297,14 @@ void* mapped_host_range(const void* host, size_t bytes) {
 // 304, 89 with all that are resident; 2^24: 807, 813 and 850 us; 2^24 of
 // N = 16: 848, 840 and 881 us.
 int64_t host_blocks(const gbfft_plan* p) {
-    const KernelEntry* e = p->entry;
+    const KernelEntry* e = p->host.entry;
     const int64_t per_block = (int64_t)e->signals_per_block * p->n * 8 * (e->pipeline > 1 ? e->pipeline : 1);
     const int64_t least = int64_t(5) << 18, most = int64_t(19) << 18;
     int64_t in_flight = p->n * p->batch / 2;  // a sixteenth of the input
     in_flight = in_flight < least ? least : in_flight > most ? most : in_flight;
     int64_t blocks = in_flight / per_block;
     if (blocks < p->sm_count / 4) blocks = p->sm_count / 4;
-    return blocks < p->resident ? blocks : p->resident;
+    return blocks < p->host.resident ? blocks : p->host.resident;
 }
 
 void release_staging(gbfft_plan* p) {
@@ -288,7 +325,7 @@ void release_staging(gbfft_plan* p) {
 // of signals), transformed in place.
 fft_status_t create_staging(gbfft_plan* p) {
     const int64_t sig_bytes = p->n * 8;
-    const int64_t S = p->entry->signals_per_block;
+    const int64_t S = p->dev.entry->signals_per_block;
     int64_t chunk = (int64_t(64) << 20) / sig_bytes;
     chunk = chunk / S * S;
     if (chunk < S) chunk = S;
@@ -441,31 +478,42 @@ fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int direction, int dty
     p->device = dev;
     p->sm_count = sms;
     p->entry = e;
-    p->kernel = direction == FFT_INVERSE ? e->kernel_inv : e->kernel_fwd;
     const bool scaled = direction == FFT_INVERSE ? !(flags & FFT_FLAG_UNNORMALIZED)
                                                  : (flags & FFT_FLAG_SCALE_FORWARD) != 0;
     p->scale = scaled ? 1.0f / (float)n : 1.0f;  // a power of two: exact
+    // Host buffers take a kernel whose grid can be bounded (host_blocks).
+    const KernelEntry* eh = nullptr;
+    if (flags & FFT_FLAG_HOST_STAGING)
+        eh = flags & FFT_FLAG_VARIANT_MASK ? e : &lv->v[default_variant(log2n, want_tc, n * batch, false)];
 
-    // twiddle table (+ error word) in one allocation
+    // twiddle tables (+ error word) in one allocation
     const size_t tw_bytes = (size_t)e->twiddles * 2 * sizeof(float);
-    const size_t alloc = tw_bytes + 256;
+    const size_t host_off = (tw_bytes + 255) / 256 * 256;
+    const size_t table_bytes = eh && eh != e ? host_off + (size_t)eh->twiddles * 2 * sizeof(float) : tw_bytes;
+    const size_t err_off = (table_bytes + 255) / 256 * 256;
     void* dmem = nullptr;
-    if (gbfft::plan_malloc(&dmem, alloc) != cudaSuccess) {
+    if (gbfft::plan_malloc(&dmem, err_off + 256) != cudaSuccess) {
         cudaGetLastError();
         delete p;
         return FFT_ERR_ALLOC;
     }
-    p->d_twiddles = (float*)dmem;
-    p->d_error = (int*)((char*)dmem + tw_bytes);
-    if (e->twiddles > 0) {
-        float* host = (float*)malloc(tw_bytes);
+    p->d_tables = dmem;
+    p->d_error = (int*)((char*)dmem + err_off);
+    const int inv = direction == FFT_INVERSE;
+    p->dev = {e, inv ? e->kernel_inv : e->kernel_fwd, (const float*)dmem, 0};
+    p->host = p->dev;
+    if (eh && eh != e)
+        p->host = {eh, inv ? eh->kernel_inv : eh->kernel_fwd, (const float*)((char*)dmem + host_off), 0};
+    if (table_bytes > 0) {
+        char* host = (char*)calloc(1, table_bytes);
         if (!host) {
             cudaFree(dmem);
             delete p;
             return FFT_ERR_ALLOC;
         }
-        e->fill_twiddles(host);
-        cudaError_t ce = cudaMemcpy(p->d_twiddles, host, tw_bytes, cudaMemcpyHostToDevice);
+        e->fill_twiddles((float*)host);
+        if (eh && eh != e) eh->fill_twiddles((float*)(host + host_off));
+        cudaError_t ce = cudaMemcpy(dmem, host, table_bytes, cudaMemcpyHostToDevice);
         free(host);
         if (ce != cudaSuccess) {
             cudaFree(dmem);
@@ -480,38 +528,18 @@ fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int direction, int dty
     }
 
     // launch shape: persistent grid, enough resident blocks to fill every SM
-    if (e->smem_bytes > 48 * 1024) {
-        if (cudaFuncSetAttribute(p->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, e->smem_bytes) !=
-            cudaSuccess) {
+    for (gbfft_plan::Launch* l : {&p->dev, &p->host}) {
+        l->resident = resident_blocks(l->entry, l->kernel, dev, sms);
+        if (l->resident < 1) {
             cudaFree(dmem);
             delete p;
-            return FFT_ERR_CUDA;
+            return l->resident < 0 ? FFT_ERR_UNSUPPORTED : FFT_ERR_CUDA;
         }
+        if (!eh || eh == e) break;
     }
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, p->kernel, e->threads_per_block,
-                                                      e->smem_bytes) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        cudaFree(dmem);
-        delete p;
-        return FFT_ERR_CUDA;
-    }
+    if (eh == e) p->host = p->dev;
     const int64_t tiles = (batch + e->signals_per_block - 1) / e->signals_per_block;
-    if (e->tmem_cols > 0) per_sm = occupancy_without_tmem(p->kernel, e->threads_per_block, e->smem_bytes, dev);
-    if (e->tmem_cols > 0 && per_sm * e->tmem_cols > 512) {
-        // every resident block holds its TMEM columns for its whole life; more
-        // than 512 per SM would leave a block waiting for columns forever
-        per_sm = 512 / e->tmem_cols;
-    }
-    if (per_sm < 1) {
-        cudaFree(dmem);
-        delete p;
-        return FFT_ERR_UNSUPPORTED;
-    }
-    const int64_t resident = (int64_t)sms * per_sm;
-    p->resident = resident;
-    p->grid = tiles < resident ? tiles : resident;
+    p->grid = tiles < p->dev.resident ? tiles : p->dev.resident;
     if ((flags & FFT_FLAG_HOST_STAGING) && batch > 0) {
         fft_status_t sst = create_staging(p);
         if (sst != FFT_OK) {
@@ -586,13 +614,13 @@ fft_status_t fft_execute_c32(fft_plan_t p, const void* in, const int8_t* in_exp,
     int64_t batch = p->batch;
     const void* in2 = in;
     void* out2 = out;
-    const float2* tw = (const float2*)p->d_twiddles;
+    const float2* tw = (const float2*)p->dev.d_twiddles;
     float scale = p->scale;
     int* err = p->d_error;
     uint64_t wait_ns = p->wait_ns;
     int stall = (p->flags & FFT_FLAG_TEST_STALL) ? 1 : 0;
     void* args[] = {&in2, &in_exp, &out2, &out_exp, &batch, &tw, &scale, &err, &wait_ns, &stall};
-    if (gbfft::launch_kernel(p->kernel, (unsigned)p->grid, (unsigned)e->threads_per_block, args,
+    if (gbfft::launch_kernel(p->dev.kernel, (unsigned)p->grid, (unsigned)e->threads_per_block, args,
                              (size_t)e->smem_bytes, (cudaStream_t)stream, batch * p->n) != cudaSuccess) {
         cudaGetLastError();
         return FFT_ERR_CUDA;
@@ -617,7 +645,7 @@ fft_status_t fft_execute(fft_plan_t p, const void* in, void* out, void* stream) 
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) return FFT_ERR_INVALID_VALUE;
 
-    return launch_plain(p, (const float2*)in, (float2*)out, p->batch, (cudaStream_t)stream, p->resident);
+    return launch_plain(p, p->dev, (const float2*)in, (float2*)out, p->batch, (cudaStream_t)stream, p->dev.resident);
 }
 
 fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host, void* stream) {
@@ -638,7 +666,7 @@ fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host,
     if (((a | b) & 15) == 0) {
         void* din = mapped_host_range(in_host, bytes);
         void* dout = a == b ? din : din ? mapped_host_range(out_host, bytes) : nullptr;
-        if (din && dout) return launch_plain(p, (const float2*)din, (float2*)dout, p->batch, user, host_blocks(p));
+        if (din && dout) return launch_plain(p, p->host, (const float2*)din, (float2*)dout, p->batch, user, host_blocks(p));
     }
     // the pipeline starts after the caller's earlier work ...
     if (cudaEventRecord(p->stage_start, user) != cudaSuccess) goto cuda_fail;
@@ -659,7 +687,7 @@ fft_status_t fft_execute_host(fft_plan_t p, const void* in_host, void* out_host,
             // order; the three streams overlap both copy directions and kernels
             if (cudaMemcpyAsync(buf, src + first * sig_bytes, nbytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
                 goto cuda_fail;
-            fft_status_t st = launch_plain(p, buf, buf, nsig, s, p->resident);
+            fft_status_t st = launch_plain(p, p->dev, buf, buf, nsig, s, p->dev.resident);
             if (st != FFT_OK) return st;
             if (cudaMemcpyAsync(dst + first * sig_bytes, buf, nbytes, cudaMemcpyDeviceToHost, s) != cudaSuccess)
                 goto cuda_fail;
@@ -711,7 +739,7 @@ fft_status_t fft_plan_get_error(fft_plan_t p) {
 fft_status_t fft_plan_destroy(fft_plan_t p) {
     if (!p) return FFT_OK;
     fft_status_t st = FFT_OK;
-    if (p->d_twiddles && cudaFree(p->d_twiddles) != cudaSuccess) st = FFT_ERR_CUDA;
+    if (p->d_tables && cudaFree(p->d_tables) != cudaSuccess) st = FFT_ERR_CUDA;
     release_staging(p);
     gbfft::ragged_destroy(p->ragged);
     delete p;
@@ -800,7 +828,7 @@ fft_status_t fft_plan_get_twiddles(fft_plan_t p, void* host_out, int64_t count) 
     if (!p || (!host_out && count > 0) || p->ragged) return FFT_ERR_INVALID_VALUE;
     if (count != p->entry->twiddles) return FFT_ERR_INVALID_VALUE;
     if (count == 0) return FFT_OK;
-    if (cudaMemcpy(host_out, p->d_twiddles, (size_t)count * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaMemcpy(host_out, p->dev.d_twiddles, (size_t)count * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
         return FFT_ERR_CUDA;
     return FFT_OK;
 }

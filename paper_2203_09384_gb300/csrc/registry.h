@@ -25,6 +25,7 @@ struct KernelEntry {
     int radix[4];
     int min_blocks;          // launch-bounds hint
     int pipeline;            // bulk-copy ring depth (0 = none)
+    bool steal;              // launched with one block per tile; running blocks take tiles of unstarted ones
     int tc;                  // 0 FP32, 1 FP16 / 2 BF16 tensor-core radix-16 stages
     int tc_stages;           // stages that run on the tensor cores
     int tmem_cols;           // TMEM columns one block allocates (tensor-core variants)

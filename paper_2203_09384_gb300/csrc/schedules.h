@@ -26,7 +26,8 @@
 //           tile placed every N + T elements of the slot (one bulk copy per
 //           signal), so that stage 0 reads them without bank conflicts,
 //      CH = cache hints: bit 0 plain loads, bit 1 plain stores (else
-//           evict-first); the defaults are the measured best per length)
+//           evict-first); bit 2: one block per tile is launched and running
+//           blocks take the tiles of blocks that have not started (TileTaker)
 // Threads per block = S * N / E.  Stage 0 with R0 = E/2 (and the last stage,
 // where its radix is E/2 or less) lets a thread own neighbouring butterflies,
 // so its HBM accesses are 128-bit.  tests/test_bank_model.py replays the
@@ -41,10 +42,10 @@
 
 #define GBFFT_GENERIC_SCHEDULES(GX)                   \
     GX(5, 1, 16, 128, 8, 4, 0, 0, 1, 0, 0, 0, 0) \
-    GX(6, 0, 16, 32, 8, 8, 0, 0, 4, 2, 0, -5, 2) \
+    GX(6, 0, 16, 16, 8, 8, 0, 0, 8, 2, 0, -5, 6) \
     GX(6, 2, 8, 32, 8, 8, 0, 0, 1, 0, 0, 3, 0) \
     GX(6, 3, 8, 32, 8, 8, 0, 0, 1, 0, 0, 0, 0) \
-    GX(7, 0, 16, 16, 8, 16, 0, 0, 4, 2, 0, -5, 2) \
+    GX(7, 0, 16, 8, 8, 16, 0, 0, 8, 2, 0, -5, 6) \
     GX(7, 1, 16, 16, 8, 16, 0, 0, 3, 2, 1, 0, 0) \
     GX(7, 2, 16, 16, 8, 16, 0, 0, 3, 2, 2, 0, 0) \
     GX(7, 3, 16, 32, 8, 16, 0, 0, 2, 0, 1, 0, 0) \
@@ -64,10 +65,10 @@
     GX(8, 14, 16, 8, 16, 16, 0, 0, 3, 2, 0, 0, 2) \
     GX(8, 15, 16, 8, 16, 16, 0, 0, 4, 2, 0, -1, 2) \
     GX(8, 16, 16, 8, 16, 16, 0, 0, 5, 2, 0, -1, 2) \
-    GX(8, 0, 16, 16, 16, 16, 0, 0, 2, 2, 0, -1, 2) \
-    GX(9, 0, 16, 8, 8, 8, 8, 0, 2, 0, 0, 0, 3) \
+    GX(8, 0, 16, 8, 16, 16, 0, 0, 4, 2, 0, -1, 6) \
+    GX(9, 0, 16, 1, 16, 2, 16, 0, 16, 2, 0, -1, 6) \
     GX(9, 1, 16, 8, 8, 8, 8, 0, 1, 0, 0, 0, 0) \
-    GX(10, 0, 16, 1, 16, 4, 16, 0, 6, 2, 0, -1, 2) \
+    GX(10, 0, 16, 1, 16, 4, 16, 0, 7, 2, 0, -1, 6) \
     GX(10, 1, 16, 2, 8, 16, 8, 0, 1, 0, 0, 0, 0) \
     GX(10, 2, 16, 2, 8, 16, 8, 0, 4, 0, 0, 0, 0) \
     GX(10, 3, 16, 2, 8, 16, 8, 0, 2, 3, 0, 0, 0) \
@@ -80,7 +81,7 @@
     GX(10, 12, 16, 2, 8, 16, 8, 0, 5, 2, 2, -2, 0) \
     GX(10, 13, 16, 2, 8, 16, 8, 0, 4, 2, 1, 1, 0) \
     GX(10, 14, 16, 2, 8, 16, 8, 0, 4, 2, 2, 1, 0) \
-    GX(11, 0, 16, 1, 16, 8, 16, 0, 3, 2, 0, -1, 2) \
+    GX(11, 0, 16, 1, 16, 8, 16, 0, 5, 2, 0, -1, 6) \
     GX(11, 1, 16, 1, 8, 16, 16, 0, 1, 0, 0, 0, 0) \
     GX(11, 2, 16, 1, 8, 16, 16, 0, 2, 3, 0, 0, 0) \
     GX(11, 3, 16, 2, 8, 16, 16, 0, 1, 2, 0, 0, 0) \
@@ -106,33 +107,41 @@
     GX(7, 8, 16, 8, 8, 16, 0, 0, 8, 0, 0, 0, 0) \
     GX(7, 9, 16, 16, 8, 16, 0, 0, 4, 2, 1, -3, 2) \
     GX(7, 10, 16, 16, 8, 16, 0, 0, 4, 2, 2, -3, 2) \
+    GX(7, 11, 16, 16, 8, 16, 0, 0, 4, 2, 1, -3, 6) \
+    GX(7, 12, 16, 16, 8, 16, 0, 0, 4, 2, 2, -3, 6) \
     GX(8, 19, 16, 4, 16, 16, 0, 0, 8, 0, 0, 0, 0) \
-    GX(8, 20, 16, 16, 16, 16, 0, 0, 2, 2, 5, -1, 2) \
+    GX(8, 20, 16, 8, 16, 16, 0, 0, 4, 2, 5, -3, 6) \
     GX(8, 21, 16, 8, 16, 16, 0, 0, 3, 2, 5, -3, 2) \
     GX(8, 22, 16, 8, 16, 16, 0, 0, 3, 2, 2, -3, 2) \
+    GX(8, 23, 16, 8, 16, 16, 0, 0, 4, 2, 2, -3, 6) \
     GX(9, 3, 16, 2, 16, 2, 16, 0, 8, 0, 0, 0, 0) \
-    GX(9, 4, 16, 4, 16, 2, 16, 0, 3, 2, 0, -1, 2) \
-    GX(10, 15, 16, 1, 16, 4, 16, 0, 6, 0, 0, 0, 0)
+    GX(10, 15, 16, 1, 16, 4, 16, 0, 6, 0, 0, 0, 0) \
+    GX(10, 16, 16, 1, 16, 4, 16, 0, 6, 2, 0, -1, 2) \
+    GX(10, 17, 16, 2, 8, 16, 8, 0, 6, 2, 1, -3, 6) \
+    GX(10, 18, 16, 2, 8, 16, 8, 0, 6, 2, 2, -3, 6) \
+    GX(11, 20, 16, 1, 16, 8, 16, 0, 3, 2, 0, -1, 2) \
+    GX(11, 21, 16, 1, 8, 16, 16, 0, 5, 2, 1, -3, 6) \
+    GX(11, 22, 16, 1, 8, 16, 16, 0, 5, 2, 2, -3, 6)
 
 #define GBFFT_SMALL_SCHEDULES(SX) \
-    SX(1, 0, 8, 1, 3)                \
+    SX(1, 0, 1, 8, 4)                \
     SX(1, 1, 8, 2, 0)                \
     SX(1, 4, 4, 2, 0)                \
-    SX(2, 0, 4, 8, 2)                \
+    SX(2, 0, 1, 4, 4)                \
     SX(2, 1, 8, 1, 0)                \
     SX(2, 2, 8, 4, 2)                \
     SX(2, 3, 16, 2, 2)               \
     SX(2, 6, 2, 2, 0)                \
-    SX(3, 0, 8, 4, 0)                \
+    SX(3, 0, 1, 2, 4)                \
     SX(3, 1, 8, 1, 0)                \
     SX(3, 2, 4, 4, 0)                \
     SX(3, 5, 4, 1, 0)                \
-    SX(4, 0, 4, 2, 2)                \
+    SX(4, 0, 1, 1, 6)                \
     SX(4, 1, 8, 1, 0)                \
     SX(4, 2, 8, 2, 0)                \
     SX(4, 5, 2, 1, 0)                \
     SX(4, 6, 2, 2, 0)                \
-    SX(5, 0, 2, 2, 0)                \
+    SX(5, 0, 1, 1, 4)                \
     SX(5, 2, 4, 1, 0)                \
     SX(5, 5, 1, 1, 0)
 
@@ -182,60 +191,71 @@
 // the last one, variant 0 (FP32) or the first variant of the type.  A default
 // set by fft_set_default_variant (the autotuner's) goes before all of this.
 //
-// Calls of up to some 12 M elements are over in a few tiles per SM: small
-// blocks and tiles spread them over more blocks, start their first store sooner
-// and leave a shorter tail, and evict-first direct loads and stores win while
-// the output still fits in L2.  Larger calls want the larger tiles of variant 0
-// (16 KB and more of consecutive bytes per copy).  Device time per call in a
-// captured graph over three rotating buffer pairs, variant 0 (as it was before
-// these rows) against the row, us:
-//   N = 2     2^21.4 9.5 / 6.6     2^23.2 26.3 / 26.2   2^24.3 53.7 / 56.0
-//   N = 4     2^21.4 8.9 / 6.8     2^23.2 28.1 / 25.6   2^24.3 53.5 / 55.8
-//   N = 8     2^16.2 3.8 / 1.6     2^22.2 17.1 / 13.0   (row 2) 2^23.6 34.1 / 32.9
-//   N = 16    2^22.2 15.8 / 13.7   2^23.2 27.1 / 25.9   (row 6) 2^24.7 68.6 / 66.3
-//   N = 32    2^20.6 5.3 / 4.5     2^22.2 14.3 / 13.0   2^24.3 53.0 / 56.4
-//   N = 64    (row 6) 2^20.6 6.4 / 4.2, 2^22.2 14.7 / 12.9   (row 5) 2^23.2 26.4 / 24.8
-//   N = 128   2^20.6 5.9 / 4.7     2^22.2 14.8 / 13.8   2^24.3 51.4 / 53.6
-//   N = 256   2^20.6 5.4 / 4.4     2^22.2 15.0 / 13.7   2^24.3 52.6 / 53.5
-//   N = 512   2^20.6 6.4 / 5.0     2^23.2 28.5 / 26.1   (row 4) 2^25.2 97.7 / 94.8, 2^28 632 / 635
-//   N = 1024  2^21.4 11.0 / 9.0    2^22.5 18.2 / 18.5
-//   N = 2048  2^21.4 11.1 / 9.8    2^21.8 13.3 / 13.5
-// The up-to-2^16 and 2^17 rows of N = 64 and 128 keep those plans on bulk-copy
-// kernels (0.3-0.8 us over the direct rows, 0.4 under variant 0).
-// Tensor-core types, rows of the same arithmetic only: FP16 N = 256 2^22.3
-// 16.1 / 14.9 (row 21), 2^28 672 / 630 (row 20); BF16 N = 256 2^24 43.7 / 41.8
-// (row 22); N = 128 2^28 672 / 638 and 655 / 643.  (Other radix orders were
-// faster still, N = 1024 and 2048 with radix 16 first and last by 2-9%, but
-// they round the operands of other stages to 16 bits.)
+// Past some 6 M elements the rows that take tiles of unstarted blocks (CH bit 2)
+// win: variant 0 at every length.  Their first request costs about 1 us, so
+// shorter calls run fixed strides, and with few tiles per SM want small blocks
+// and tiles, which start their first store sooner and leave a shorter tail;
+// evict-first direct loads and stores win while the output still fits in L2.
+// Device time per call in a captured graph over three rotating buffer pairs, us:
+// the best single schedule for all sizes that these rows replaced / the row for
+// short calls / variant 0:
+//   N = 2     2^21.4  9.5 /  6.6 /  -     2^22.2 14.4 / 13.0 / 12.8   2^24 44.1 / 45.3 / 40.5   2^28 652 / 606
+//   N = 4     2^21.4  8.9 /  6.8 /  -     2^22.2 16.1 / 12.9 / 13.0   2^24 44.7 / 45.3 / 40.6   2^28 650 / 606
+//   N = 8     2^21.4  9.5 /  7.0 /  -     2^22.2 17.1 / 13.0 / 13.1   2^24 43.6 / 45.6 / 40.7   2^28 652 / 606
+//   N = 16    2^21.4  8.8 /  7.3 /  -     2^22.2 15.8 / 13.7 / 13.0   2^24 43.6 / 45.4 / 40.7   2^28 650 / 610
+//   N = 32    2^21.4 10.7 /  8.2 /  -     2^22.2 14.3 / 13.0 / 13.1   2^24 43.9 / 45.0 / 40.7   2^28 645 / 606
+//   N = 64    2^21.4 10.4 /  7.6 /  -     2^22.2 14.7 / 12.9 / 13.8   2^24 43.5 / 46.4 / 39.8   2^28 631 / 600
+//   N = 128   2^21.4 10.8 /  8.5 /  -     2^22.2 14.8 / 13.7 / 14.1   2^24 42.6 / 43.4 / 40.3   2^28 633 / 601
+//   N = 256   2^21.4 10.7 /  8.4 /  -     2^22.2 15.0 / 13.7 / 14.0   2^24 43.2 / 43.2 / 41.1   2^28 642 / 602
+//   N = 512   2^21.4 12.1 /  8.7 /  -     2^22.2 16.2 / 14.4 / 15.4   2^24 45.2 / 43.4 / 41.9   2^28 636 / 603
+//   N = 1024  2^21.4 11.8 /  9.0 /  -     2^22.2 17.3 / 15.5 / 16.4   2^24 45.6 / 43.4 / 41.9   2^28 650 / 602
+//   N = 2048  2^21.4 12.0 /  9.8 / 12.9   2^23.2 28.7 / 27.4 / 28.0   2^24 45.7 / 44.5 / 44.0   2^28 652 / 607
+// The rows up to 2^16 and 2^17 of N = 64 and 128 keep those plans on bulk-copy
+// kernels (0.3-0.8 us over the direct rows, 0.4 under the earlier default).
+//
+// Tensor-core types: every row of a length rounds the same operands.  Before /
+// after at 2^28: FP16 N = 128 672 / 607, 256 666 / 600, 1024 727 / 686,
+// 2048 681 / 643; BF16 655 / 603, 643 / 600, 704 / 660, 665 / 632.  (Radix 16
+// first and last was faster still by 2-9% at 1024 and 2048, but rounds other
+// stages' operands to 16 bits.)
 #define GBFFT_SIZE_DEFAULTS(DX) \
-    DX(1, 0, 8 << 20, 4)        \
-    DX(2, 0, 12 << 20, 6)       \
-    DX(3, 0, 8 << 20, 5)        \
-    DX(3, 0, 12 << 20, 2)       \
-    DX(4, 0, 12 << 20, 5)       \
-    DX(4, 0, 30 << 20, 6)       \
-    DX(5, 0, 12 << 20, 5)       \
+    DX(1, 0, 5 << 20, 4)        \
+    DX(2, 0, 5 << 20, 6)        \
+    DX(3, 0, 5 << 20, 5)        \
+    DX(4, 0, 4 << 20, 5)        \
+    DX(5, 0, 5 << 20, 5)        \
     DX(6, 0, 1 << 16, 5)        \
     DX(6, 0, 6 << 20, 6)        \
-    DX(6, 0, 16 << 20, 5)       \
     DX(7, 0, 1 << 17, 7)        \
-    DX(7, 0, 12 << 20, 8)       \
-    DX(8, 0, 16 << 20, 19)      \
-    DX(9, 0, 20 << 20, 3)       \
-    DX(9, 0, 160 << 20, 4)      \
-    DX(10, 0, 1 << 20, 0)       \
+    DX(7, 0, 6 << 20, 8)        \
+    DX(8, 0, 6 << 20, 19)       \
+    DX(9, 0, 6 << 20, 3)        \
+    DX(10, 0, 1 << 20, 16)      \
     DX(10, 0, 5 << 20, 15)      \
-    DX(11, 0, 3 << 19, 0)       \
+    DX(10, 0, 7 << 20, 16)      \
+    DX(11, 0, 3 << 19, 20)      \
     DX(11, 0, 3 << 20, 1)       \
+    DX(11, 0, 12 << 20, 20)     \
     DX(7, 1, 2 << 20, 1)        \
-    DX(7, 1, INT64_MAX, 9)      \
+    DX(7, 1, 16 << 20, 9)       \
+    DX(7, 1, INT64_MAX, 11)     \
     DX(7, 2, 2 << 20, 2)        \
-    DX(7, 2, INT64_MAX, 10)     \
+    DX(7, 2, 16 << 20, 10)      \
+    DX(7, 2, INT64_MAX, 12)     \
     DX(8, 1, 2 << 20, 1)        \
-    DX(8, 1, 24 << 20, 21)      \
+    DX(8, 1, 12 << 20, 21)      \
     DX(8, 1, INT64_MAX, 20)     \
     DX(8, 2, 1 << 19, 2)        \
-    DX(8, 2, 24 << 20, 22)
+    DX(8, 2, 12 << 20, 22)      \
+    DX(8, 2, INT64_MAX, 23)     \
+    DX(10, 1, 20 << 20, 4)      \
+    DX(10, 1, INT64_MAX, 17)    \
+    DX(10, 2, 20 << 20, 5)      \
+    DX(10, 2, INT64_MAX, 18)    \
+    DX(11, 1, 20 << 20, 4)      \
+    DX(11, 1, INT64_MAX, 21)    \
+    DX(11, 2, 20 << 20, 5)      \
+    DX(11, 2, INT64_MAX, 22)
 
 #define GBFFT_MIN_LOG2N 1
 #define GBFFT_MAX_LOG2N 11
