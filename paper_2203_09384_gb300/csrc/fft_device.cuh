@@ -1766,92 +1766,130 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
 // warp's shared-memory slab in 128-bit pieces (4 elements each); each lane
 // finds its own signal's exponent without any exchange.
 template <class SC, bool INV>
+__device__ __forceinline__ void small_c32_tile(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp,
+                                               int64_t batch, int ls, float4* sm, int64_t wt) {
+    constexpr int N = SC::N, U = SC::UNROLL;
+    constexpr int TS = 32 * U;         // signals per warp tile
+    constexpr int P = TS * N / 4;      // 128-bit pieces per warp tile
+    const int lane = threadIdx.x & 31;
+    const int64_t first = wt * TS;
+    const int64_t left = batch - first;
+    const int nsig = (int)(left < TS ? left : TS);
+    const int valid_e = nsig * N;          // binary16 pairs in this tile
+    const int full = valid_e / 4;          // whole 128-bit pieces
+    const float4* src = reinterpret_cast<const float4*>(in + first * N);
+    float4* dst = reinterpret_cast<float4*>(out + first * N);
+#pragma unroll
+    for (int i = 0; i < (P + 31) / 32; ++i) {
+        const int p = lane + 32 * i;
+        if (p < full) sm[swz16<N>(p)] = ld_stream4v<SC::CH>(src + p);
+    }
+    if (N == 2 && lane == 0 && (valid_e & 3))  // odd signal count: the last signal is half a piece
+        reinterpret_cast<float2*>(sm + swz16<N>(full))[0] =
+            *reinterpret_cast<const float2*>(in + first * N + 4 * full);
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int sg = u * 32 + lane;
+        const bool act = sg < nsig;
+        const int ein = act ? (int)in_exp[first + sg] : 0;
+        float2 v[N];
+        if constexpr (N >= 4) {
+#pragma unroll
+            for (int i = 0; i < N / 4; ++i) {
+                const float4 f = sm[swz16<N>(sg * (N / 4) + i)];
+                v[4 * i + 0] = __half22float2(bits_h2(f.x));
+                v[4 * i + 1] = __half22float2(bits_h2(f.y));
+                v[4 * i + 2] = __half22float2(bits_h2(f.z));
+                v[4 * i + 3] = __half22float2(bits_h2(f.w));
+            }
+        } else {
+            const float2 f = reinterpret_cast<const float2*>(sm + swz16<N>(sg >> 1))[sg & 1];
+            v[0] = __half22float2(bits_h2(f.x));
+            v[1] = __half22float2(bits_h2(f.y));
+        }
+        if constexpr (INV) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) v[i].y = -v[i].y;
+        }
+        Dft<N>::run(v);
+        float m = 0.0f;
+#pragma unroll
+        for (int i = 0; i < N; ++i) m = fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
+        const C32Out o = c32_out_scale<N>(m, ein, ls);
+        const float my = INV ? -o.mult : o.mult;
+        float hw[N];  // binary16 pairs as 32-bit words
+#pragma unroll
+        for (int i = 0; i < N; ++i) hw[i] = h2_bits(__floats2half2_rn(v[i].x * o.mult, v[i].y * my));
+        if constexpr (N >= 4) {
+#pragma unroll
+            for (int i = 0; i < N / 4; ++i)
+                sm[swz16<N>(sg * (N / 4) + i)] = make_float4(hw[4 * i], hw[4 * i + 1], hw[4 * i + 2], hw[4 * i + 3]);
+        } else {
+            reinterpret_cast<float2*>(sm + swz16<N>(sg >> 1))[sg & 1] = make_float2(hw[0], hw[1]);
+        }
+        if (act) out_exp[first + sg] = (int8_t)o.e;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < (P + 31) / 32; ++i) {
+        const int p = lane + 32 * i;
+        if (p < full) st_stream4v<SC::CH>(dst + p, sm[swz16<N>(p)]);
+    }
+    if (N == 2 && lane == 0 && (valid_e & 3))
+        *reinterpret_cast<float2*>(out + first * N + 4 * full) = reinterpret_cast<const float2*>(sm + swz16<N>(full))[0];
+    __syncwarp();
+}
+
+template <class SC, bool INV>
 __global__ void __launch_bounds__(SC::NT)
     fft_small_c32_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp, int64_t batch,
                          const float2* __restrict__ tw, float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
-    constexpr int N = SC::N, W = SC::WARPS_PER_BLOCK, U = SC::UNROLL;
-    constexpr int TS = 32 * U;         // signals per warp tile
-    constexpr int P = TS * N / 4;      // 128-bit pieces per warp tile
+    constexpr int W = SC::WARPS_PER_BLOCK, TS = 32 * SC::UNROLL, P = TS * SC::N / 4;
     extern __shared__ __align__(16) float4 smem4[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float4* sm = smem4 + warp * P;
+    const int warp = threadIdx.x >> 5;
     const int ls = log2_pow2(scale);
     const int64_t wtiles = (batch + TS - 1) / TS;
-    for (int64_t wt = (int64_t)blockIdx.x * W + warp; wt < wtiles; wt += (int64_t)gridDim.x * W) {
-        const int64_t first = wt * TS;
-        const int64_t left = batch - first;
-        const int nsig = (int)(left < TS ? left : TS);
-        const int valid_e = nsig * N;          // binary16 pairs in this tile
-        const int full = valid_e / 4;          // whole 128-bit pieces
-        const float4* src = reinterpret_cast<const float4*>(in + first * N);
-        float4* dst = reinterpret_cast<float4*>(out + first * N);
-#pragma unroll
-        for (int i = 0; i < (P + 31) / 32; ++i) {
-            const int p = lane + 32 * i;
-            if (p < full) sm[swz16<N>(p)] = ld_stream4v<SC::CH>(src + p);
-        }
-        if (N == 2 && lane == 0 && (valid_e & 3))  // odd signal count: the last signal is half a piece
-            reinterpret_cast<float2*>(sm + swz16<N>(full))[0] =
-                *reinterpret_cast<const float2*>(in + first * N + 4 * full);
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int sg = u * 32 + lane;
-            const bool act = sg < nsig;
-            const int ein = act ? (int)in_exp[first + sg] : 0;
-            float2 v[N];
-            if constexpr (N >= 4) {
-#pragma unroll
-                for (int i = 0; i < N / 4; ++i) {
-                    const float4 f = sm[swz16<N>(sg * (N / 4) + i)];
-                    v[4 * i + 0] = __half22float2(bits_h2(f.x));
-                    v[4 * i + 1] = __half22float2(bits_h2(f.y));
-                    v[4 * i + 2] = __half22float2(bits_h2(f.z));
-                    v[4 * i + 3] = __half22float2(bits_h2(f.w));
-                }
-            } else {
-                const float2 f = reinterpret_cast<const float2*>(sm + swz16<N>(sg >> 1))[sg & 1];
-                v[0] = __half22float2(bits_h2(f.x));
-                v[1] = __half22float2(bits_h2(f.y));
-            }
-            if constexpr (INV) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) v[i].y = -v[i].y;
-            }
-            Dft<N>::run(v);
-            float m = 0.0f;
-#pragma unroll
-            for (int i = 0; i < N; ++i) m = fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-            const C32Out o = c32_out_scale<N>(m, ein, ls);
-            const float my = INV ? -o.mult : o.mult;
-            float hw[N];  // binary16 pairs as 32-bit words
-#pragma unroll
-            for (int i = 0; i < N; ++i) hw[i] = h2_bits(__floats2half2_rn(v[i].x * o.mult, v[i].y * my));
-            if constexpr (N >= 4) {
-#pragma unroll
-                for (int i = 0; i < N / 4; ++i)
-                    sm[swz16<N>(sg * (N / 4) + i)] = make_float4(hw[4 * i], hw[4 * i + 1], hw[4 * i + 2], hw[4 * i + 3]);
-            } else {
-                reinterpret_cast<float2*>(sm + swz16<N>(sg >> 1))[sg & 1] = make_float2(hw[0], hw[1]);
-            }
-            if (act) out_exp[first + sg] = (int8_t)o.e;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < (P + 31) / 32; ++i) {
-            const int p = lane + 32 * i;
-            if (p < full) st_stream4v<SC::CH>(dst + p, sm[swz16<N>(p)]);
-        }
-        if (N == 2 && lane == 0 && (valid_e & 3))
-            *reinterpret_cast<float2*>(out + first * N + 4 * full) = reinterpret_cast<const float2*>(sm + swz16<N>(full))[0];
-        __syncwarp();
+    for (int64_t wt = (int64_t)blockIdx.x * W + warp; wt < wtiles; wt += (int64_t)gridDim.x * W)
+        small_c32_tile<SC, INV>(in, in_exp, out, out_exp, batch, ls, smem4 + warp * P, wt);
+}
+
+// The same with one warp per block, taking the tiles of unstarted blocks, as
+// in fft_small_steal_kernel.
+template <class SC, bool INV>
+__global__ void __launch_bounds__(SC::NT)
+    fft_small_c32_steal_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp, int64_t batch,
+                               const float2* __restrict__ tw, float scale, int* err, uint64_t wait_ns, int stall) {
+    pdl_enter();
+    extern __shared__ __align__(16) float4 smem4[];
+    unsigned char* steal = reinterpret_cast<unsigned char*>(smem4) + SC::kSlabBytes;
+    const int ls = log2_pow2(scale);
+    TileTaker taker;  // lane 0's requests
+    if (threadIdx.x == 0) {
+        taker.resp = steal;
+        taker.bar = reinterpret_cast<uint64_t*>(steal + 16);
+        mbar_init(taker.bar, 1);
+        fence_mbar_init();
+        taker.request();
     }
+    for (int64_t tile = blockIdx.x; tile >= 0;) {
+        small_c32_tile<SC, INV>(in, in_exp, out, out_exp, batch, ls, smem4, tile);
+        if (threadIdx.x == 0) {
+            bool late = false;
+            tile = taker.take(wait_ns, late);
+            if (late) atomicCAS(err, 0, kErrTimeout);
+            if (tile >= 0) taker.request();
+        }
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+    }
+    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up
 }
 
 template <int LOG2N, int WARPS, int U = 1, int CH_ = 0>
 struct SmallC32Cfg : SmallCfg<LOG2N, WARPS, U, CH_> {
-    static constexpr int kSmemBytes = WARPS * 32 * U * (1 << LOG2N) * 4;
+    static constexpr int kSlabBytes = WARPS * 32 * U * (1 << LOG2N) * 4;
+    static constexpr int kSmemBytes = kSlabBytes + (SmallCfg<LOG2N, WARPS, U, CH_>::kSteal ? 32 : 0);
 };
 
 }  // namespace gbfft

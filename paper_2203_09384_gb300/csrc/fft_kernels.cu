@@ -74,7 +74,7 @@ static KernelEntry c32_entry(int variant) {
     return e;
 }
 
-// two signals per thread (XB = 6)
+// two signals per thread (XB = 6, 14)
 template <class C>
 static KernelEntry pair_c32_entry(int variant) {
     KernelEntry e{};
@@ -89,6 +89,7 @@ static KernelEntry pair_c32_entry(int variant) {
     for (int s = 0; s < 4; ++s) e.radix[s] = C::radix(s);
     e.min_blocks = C::MINB;
     e.pipeline = C::D;
+    e.steal = C::kSteal;
     e.twiddles = C::kTwiddles;
     if constexpr (C::kWarpLocal) {
         e.kernel_fwd = reinterpret_cast<const void*>(&fft_pair_c32_warp_kernel<C, false>);
@@ -103,8 +104,8 @@ static KernelEntry pair_c32_entry(int variant) {
 
 template <int L, int E, int S, int R0, int R1, int R2, int R3, int MINB, int PIPE, int XB>
 static KernelEntry c32_row(int variant) {
-    if constexpr (XB == 6) {
-        return pair_c32_entry<PairCfg<L, E, S, R0, R1, R2, R3, MINB, PIPE>>(variant);
+    if constexpr ((XB & 7) == 6) {
+        return pair_c32_entry<PairCfg<L, E, S, R0, R1, R2, R3, MINB, PIPE, (XB & 8) != 0>>(variant);
     } else {
         static_assert(PIPE == 0, "one signal per thread group: direct loads");
         return c32_entry<Cfg<L, E, S, R0, R1, R2, R3, MINB, 0, 0, XB, 0>>(variant);
@@ -126,8 +127,14 @@ static KernelEntry small_c32_entry(int variant) {
     e.radix[0] = SC::N;
     e.min_blocks = 1;
     e.twiddles = 0;
-    e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_c32_kernel<SC, false>);
-    e.kernel_inv = reinterpret_cast<const void*>(&fft_small_c32_kernel<SC, true>);
+    e.steal = SC::kSteal;
+    if constexpr (SC::kSteal) {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_c32_steal_kernel<SC, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_small_c32_steal_kernel<SC, true>);
+    } else {
+        e.kernel_fwd = reinterpret_cast<const void*>(&fft_small_c32_kernel<SC, false>);
+        e.kernel_inv = reinterpret_cast<const void*>(&fft_small_c32_kernel<SC, true>);
+    }
     e.fill_twiddles = &fill_nothing;
     return e;
 }

@@ -150,8 +150,11 @@ struct PairDft<16> {
 // threads per pair, a ring of D tiles filled by bulk copies (per warp when a
 // pair lives in one warp, per block when it spans warps)
 // ---------------------------------------------------------------------------
-template <int LOG2N_, int E_, int S_, int R0, int R1, int R2, int R3, int MINB_, int D_>
+template <int LOG2N_, int E_, int S_, int R0, int R1, int R2, int R3, int MINB_, int D_, bool STEAL_>
 struct PairCfg {
+    // one block per tile is launched, and a running block takes the tiles of
+    // blocks that have not started (TileTaker)
+    static constexpr bool kSteal = STEAL_;
     static constexpr int LOG2N = LOG2N_;
     static constexpr int N = 1 << LOG2N_;
     static constexpr int E = E_;
@@ -184,7 +187,9 @@ struct PairCfg {
     static constexpr int kUnitBytes = kExchangeBytes + D * kSlotBytes;
     static constexpr int kBarOffset = kUnits * kUnitBytes;
     static constexpr int kRedOffset = kBarOffset + kUnits * D * 8;
-    static constexpr int kSmemBytes = kWarpLocal ? kRedOffset : kRedOffset + 2 * (NT / 32) * 4;
+    // tile stealing: the answer, its mbarrier, the tile in the slot (-1: no more)
+    static constexpr int kStealOffset = (kRedOffset + (kWarpLocal ? 0 : 2 * (NT / 32) * 4) + 15) / 16 * 16;
+    static constexpr int kSmemBytes = kSteal ? kStealOffset + 32 : kStealOffset;
     // A tile in shared memory is split into groups of consecutive signals
     // placed 128 / groups bytes apart, and neighbouring pairs of a warp take
     // their signals from different groups: one access of the warp (stage s:
@@ -194,6 +199,7 @@ struct PairCfg {
         return !kWarpLocal ? 1 : E / radix(s) >= 2 ? (16 / T > 1 ? 16 / T : 1) : (32 / T > 1 ? 32 / T : 1);
     }
     static_assert(ns(M) == N && S % 2 == 0 && NT % 32 == 0 && D >= 1, "whole pairs, whole warps");
+    static_assert(!kSteal || (kUnits == 1 && D == 1), "tile stealing: one tile at a time per block, one slot");
     static_assert(E % R0 == 0 && E % (R1 ? R1 : 1) == 0 && E % (R2 ? R2 : 1) == 0 && E % (R3 ? R3 : 1) == 0,
                   "every radix must divide E");
 };
@@ -427,6 +433,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     dbg_set_err(err);
 
     RingInFlight inflight;  // lane 0's copies in flight
+    TileTaker taker;        // lane 0's requests (kSteal)
     // lane 0: tile `tile` into `slot`; the tile of the warp's iteration j goes to slot j mod D
     auto issue = [&](int slot, int64_t tile, uint32_t parity) {
         const int64_t first = tile * C::SU;
@@ -447,6 +454,11 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     };
     if (lane == 0) {
         for (int d = 0; d < D; ++d) mbar_init(&bars[d], 1);
+        if constexpr (C::kSteal) {
+            taker.resp = base8 + C::kStealOffset;
+            taker.bar = reinterpret_cast<uint64_t*>(base8 + C::kStealOffset + 16);
+            mbar_init(taker.bar, 1);
+        }
         fence_mbar_init();
     }
     __syncwarp();
@@ -454,6 +466,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         for (int d = 0; d < D; ++d)
             if (first_tile + d * step < ntiles) issue(d, first_tile + d * step, 0);
     }
+    if (C::kSteal && lane == 0) taker.request();
     bool dead = false;
     if (stall) {  // failure-detection test mode: a phase nothing will complete
         if (!mbar_wait_bounded(&bars[0], 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
@@ -462,7 +475,8 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     const int own = pair_signal<C, GI>(pr);  // the thread's first signal in the tile
     int slot = 0;
     uint32_t parity = 0;  // of the slot's current use
-    for (int64_t tile = first_tile; tile < ntiles; tile += step) {
+    int64_t next = 0;  // kSteal: the tile after this one, or -1
+    for (int64_t tile = first_tile; tile >= 0 && tile < ntiles; tile = C::kSteal ? next : tile + step) {
         const int64_t first = tile * C::SU;
         const int64_t sig = first + own;
         const bool in_a = sig < batch, in_b = sig + 1 < batch;
@@ -475,6 +489,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
                 atomicCAS(err, 0, kErrTimeout);
             }
         }
+        if (C::kSteal && __any_sync(0xffffffffu, dead)) break;
         C2 v[C::E];
         pair_load<C, INV>(v, reinterpret_cast<const uint32_t*>(ring + slot * C::kSlotBytes) + pair_place<C, GI>(own), t);
         // the slot has been read: refill it; and the previous tile's copy out
@@ -482,9 +497,20 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-            if (!dead && !stall && tile + D * step < ntiles) issue(slot, tile + D * step, parity ^ 1);
+            if constexpr (C::kSteal) {
+                bool late = false;
+                next = taker.take(wait_ns, late);
+                if (late) atomicCAS(err, 0, kErrTimeout);
+                if (next >= 0) {
+                    issue(slot, next, parity ^ 1);
+                    taker.request();
+                }
+            } else {
+                if (!dead && !stall && tile + D * step < ntiles) issue(slot, tile + D * step, parity ^ 1);
+            }
             bulk_wait_read();
         }
+        if constexpr (C::kSteal) next = __shfl_sync(0xffffffffu, next, 0);
         if (++slot == D) {
             slot = 0;
             parity ^= 1;
@@ -520,6 +546,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     }
     if (lane == 0) {
         bulk_wait_all();
+        if constexpr (C::kSteal) taker.drain(wait_ns);
         inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
     }
 }
@@ -546,35 +573,41 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     dbg_set_err(err);
 
     RingInFlight inflight;  // thread 0's copies in flight
-    auto issue = [&](int64_t j) {  // the block's tile of iteration j into slot j mod D (thread 0 only)
-        const int slot = (int)(j % D);
-        const int64_t first = (blockIdx.x + j * gridDim.x) * C::S;
+    TileTaker taker;        // thread 0's requests (kSteal)
+    volatile int64_t* slot_tile = reinterpret_cast<volatile int64_t*>(base8 + C::kStealOffset + 24);  // kSteal
+    // thread 0: `tile` into `slot`, for its use with phase parity `parity`
+    auto issue = [&](int slot, int64_t tile, uint32_t parity) {
+        const int64_t first = tile * C::S;
         const int64_t left = batch - first;
         const uint32_t bytes = (uint32_t)((left < C::S ? left : C::S) * C::N * 4);
+        if constexpr (C::kSteal) *slot_tile = tile;
         mbar_arrive_expect_tx(&bars[slot], bytes);
         bulk_copy_g2s(base8 + C::kExchangeBytes + slot * C::kSlotBytes, in + first * C::N, bytes, &bars[slot]);
-        inflight.issued(slot, (uint32_t)((j / D) & 1));
+        inflight.issued(slot, parity);
     };
     if (tid == 0) {
         for (int d = 0; d < D; ++d) mbar_init(&bars[d], 1);
+        if constexpr (C::kSteal) {
+            taker.resp = base8 + C::kStealOffset;
+            taker.bar = reinterpret_cast<uint64_t*>(base8 + C::kStealOffset + 16);
+            mbar_init(taker.bar, 1);
+        }
         fence_mbar_init();
     }
     __syncthreads();
     if (tid == 0 && !stall) {
         for (int d = 0; d < D; ++d)
-            if (blockIdx.x + (int64_t)d * gridDim.x < ntiles) issue(d);
+            if (blockIdx.x + (int64_t)d * gridDim.x < ntiles) issue(d, blockIdx.x + (int64_t)d * gridDim.x, 0);
     }
+    if (C::kSteal && tid == 0) taker.request();
     bool dead = false;
     if (stall) {  // failure-detection test mode: a phase nothing will complete
         if (!mbar_wait_bounded(&bars[0], 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         dead = true;
     }
     int64_t it = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+    for (int64_t tile = blockIdx.x; C::kSteal || tile < ntiles; tile += gridDim.x, ++it) {
         const int slot = (int)(it % D);
-        const int64_t sig = tile * C::S + 2 * pr;
-        const bool in_a = sig < batch, in_b = sig + 1 < batch;
-        const int ea = in_a ? (int)in_exp[sig] : 0, eb = in_b ? (int)in_exp[sig + 1] : 0;
         if (!dead) {
             if (mbar_wait_bounded(&bars[slot], (uint32_t)((it / D) & 1), wait_ns)) {
                 inflight.completed(slot);
@@ -583,6 +616,17 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
                 atomicCAS(err, 0, kErrTimeout);
             }
         }
+        if constexpr (C::kSteal) {
+            tile = dead ? -1 : *slot_tile;
+            // every thread leaves in the same iteration, also when one gave up
+            if (tile < 0) {
+                __syncthreads_or(dead);
+                break;
+            }
+        }
+        const int64_t sig = tile * C::S + 2 * pr;
+        const bool in_a = sig < batch, in_b = sig + 1 < batch;
+        const int ea = in_a ? (int)in_exp[sig] : 0, eb = in_b ? (int)in_exp[sig + 1] : 0;
         const uint32_t* src =
             reinterpret_cast<const uint32_t*>(base8 + C::kExchangeBytes + slot * C::kSlotBytes) + 2 * pr * C::N;
         C2 v[C::E];
@@ -591,8 +635,26 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         // (the previous tile's barrier before its store: the exchange buffer has been read)
         pair_scatter<C, 0>(v, smem4, pr * C::N, t);
         fence_proxy_async_smem();
-        __syncthreads();  // ... and every thread has read the slot: refill it
-        if (tid == 0 && !dead && !stall && tile + (int64_t)D * gridDim.x < ntiles) issue(it + D);
+        // ... and every thread has read the slot: refill it
+        if constexpr (C::kSteal) {
+            if (__syncthreads_or(dead)) break;
+            if (tid == 0) {
+                bool late = false;
+                const int64_t next = taker.take(wait_ns, late);
+                if (late) atomicCAS(err, 0, kErrTimeout);
+                if (next >= 0) {
+                    issue(slot, next, (uint32_t)((it + 1) & 1));
+                    taker.request();
+                } else {
+                    *slot_tile = -1;
+                    mbar_arrive(&bars[slot]);
+                }
+            }
+        } else {
+            __syncthreads();
+            if (tid == 0 && !dead && !stall && tile + (int64_t)D * gridDim.x < ntiles)
+                issue(slot, tile + (int64_t)D * gridDim.x, (uint32_t)((it / D + 1) & 1));
+        }
         pair_gather<C, 1>(v, smem4, pr * C::N, t);
         pair_twist_dft<C, 1>(v, t, tw);
         pair_stages<C, 2>(v, smem4, pr * C::N, t, tw);
@@ -613,7 +675,10 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         if (t == 0 && act_b) out_exp[sig + 1] = (int8_t)ob.e;
         pair_store<C, INV, true>(v, out + sig * C::N, t, act_a, act_b, oa.mult, ob.mult);
     }
-    if (tid == 0) inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
+    if (tid == 0) {
+        if constexpr (C::kSteal) taker.drain(wait_ns);
+        inflight.drain(bars, wait_ns);  // copies in flight after a wait gave up
+    }
 }
 
 }  // namespace gbfft

@@ -60,8 +60,9 @@ LengthVariants* registry() {
 }
 
 // The variant of a plan that names none: type `tc` (0 FP32, 1 FP16 / 2 BF16
-// tensor cores), calls of `elems` elements.  Without `steal`, the last row for
+// tensor cores, 3 complex32), calls of `elems` elements.  Without `steal`, the last row for
 // smaller calls in place of one that needs a block per tile.
+constexpr int kTcC32 = 3;
 int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
     struct Row {
         int log2n, tc;
@@ -73,7 +74,9 @@ int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
 #undef GBFFT_DX
     const LengthVariants& lv = registry()[log2n];
     int fallback = 0;
-    if (tc != 0) {
+    if (tc == kTcC32) {
+        while (lv.v[fallback].kind != KernelKind::C32) ++fallback;  // every length has one
+    } else if (tc != 0) {
         while (fallback < lv.count && lv.v[fallback].tc != tc) ++fallback;
         if (fallback == lv.count) return default_variant(log2n, 0, elems, steal);  // no radix-16 stage: FP32
     } else if (const int preferred = lv.preferred.load()) {
@@ -455,13 +458,8 @@ fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int direction, int dty
     const bool want_c32 = dtype == FFT_C32;
     int variant = (int)((flags & FFT_FLAG_VARIANT_MASK) >> 8) - 1;
     if (variant < 0) {
-        // complex32 storage: the first complex32 variant.  Otherwise by size;
-        // lengths without a tensor-core schedule run FP32.
-        if (want_c32) {
-            for (variant = 0; lv->v[variant].kind != KernelKind::C32;) ++variant;  // every length has one
-        } else {
-            variant = default_variant(log2n, want_tc, n * batch);
-        }
+        // by size; lengths without a tensor-core schedule run FP32
+        variant = default_variant(log2n, want_c32 ? kTcC32 : want_tc, n * batch);
     }
     if (variant >= lv->count || !lv->v[variant].kernel_fwd) return FFT_ERR_INVALID_VALUE;
     if (lv->v[variant].tc != 0 && lv->v[variant].tc != want_tc) return FFT_ERR_INVALID_VALUE;
@@ -620,7 +618,8 @@ fft_status_t fft_execute_c32(fft_plan_t p, const void* in, const int8_t* in_exp,
     uint64_t wait_ns = p->wait_ns;
     int stall = (p->flags & FFT_FLAG_TEST_STALL) ? 1 : 0;
     void* args[] = {&in2, &in_exp, &out2, &out_exp, &batch, &tw, &scale, &err, &wait_ns, &stall};
-    if (gbfft::launch_kernel(p->dev.kernel, (unsigned)p->grid, (unsigned)e->threads_per_block, args,
+    const int64_t grid = e->steal ? (batch + e->signals_per_block - 1) / e->signals_per_block : p->grid;
+    if (gbfft::launch_kernel(p->dev.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
                              (size_t)e->smem_bytes, (cudaStream_t)stream, batch * p->n) != cudaSuccess) {
         cudaGetLastError();
         return FFT_ERR_CUDA;

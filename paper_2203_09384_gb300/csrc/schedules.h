@@ -148,7 +148,8 @@
 // complex32-storage rows (FFT_C32): CX(log2N, variant, E, S, R0..R3, MINB,
 // PIPE, XB).  XB = 6 (N >= 64): two signals per thread, packed FP32 arithmetic
 // (fft_pair.cuh), S / 2 signal pairs and S N / (2 E) threads per block, a ring
-// of PIPE bulk-copied tiles per warp (N <= 512) or per block.  XB = 0: the
+// of PIPE bulk-copied tiles per warp (N <= 512) or per block; XB = 14: the same,
+// taking the tiles of unstarted blocks (one warp per block for N <= 512).  XB = 0: the
 // Stockham kernel with binary16 loads/stores, one signal per thread group.
 // A length's first complex32 row is its default; for N <= 32 that is the
 // one-thread-per-signal SCX row further down.
@@ -156,7 +157,8 @@
 // Why the defaults are shaped so (2^27 elements, device time, against the
 // one-signal-per-thread kernels they replaced, whose stored values and
 // exponents they reproduce bit for bit): N = 64 244 -> 169 us, 128 241 -> 178,
-// 256 210 -> 180, 512 285 -> 208, 1024 303 -> 220, 2048 302 -> 239.  Blocks of
+// 256 210 -> 180, 512 285 -> 208, 1024 303 -> 220, 2048 302 -> 239 (and with
+// tiles taken from unstarted blocks 164, 169, 169, -, 213, 232).  Blocks of
 // 64 threads at N = 1024 (128: 237 us), because its barriers then join two
 // warps only; one ring slot, because a second one costs the fourth block per SM
 // (N = 1024 and 2048: 252 and 262 us with two slots and three blocks).
@@ -175,7 +177,12 @@
     CX(10, 9, 16, 4, 8, 16, 8, 0, 4, 1, 6)       \
     CX(11, 8, 16, 2, 8, 16, 16, 0, 4, 1, 6)      \
     CX(11, 9, 16, 2, 8, 16, 16, 0, 3, 2, 6)      \
-    CX(8, 5, 16, 16, 16, 16, 0, 0, 4, 1, 6)
+    CX(8, 5, 16, 16, 16, 16, 0, 0, 4, 1, 6)      \
+    CX(6, 7, 16, 16, 8, 8, 0, 0, 16, 1, 14)      \
+    CX(7, 13, 16, 8, 8, 16, 0, 0, 16, 1, 14)     \
+    CX(8, 24, 16, 4, 16, 16, 0, 0, 16, 1, 14)    \
+    CX(10, 19, 16, 2, 8, 16, 8, 0, 8, 1, 14)     \
+    CX(11, 23, 16, 2, 8, 16, 16, 0, 4, 1, 14)
 
 // complex32 one-thread-per-signal rows (N <= 32): SCX(log2N, variant, warps
 // per block, 32-signal groups per warp tile, cache hints)
@@ -184,10 +191,15 @@
     SCX(2, 4, 4, 8, 0)                  \
     SCX(3, 3, 8, 4, 0)                  \
     SCX(4, 3, 4, 4, 0)                  \
-    SCX(5, 3, 4, 2, 0)
+    SCX(5, 3, 4, 2, 0)                  \
+    SCX(2, 7, 1, 4, 4)                  \
+    SCX(3, 6, 1, 4, 4)                  \
+    SCX(4, 7, 1, 2, 4)                  \
+    SCX(5, 6, 1, 1, 4)
 
 // Which row a plan that names none runs, by length, type and size of the call:
-// DX(log2N, tc type, largest n * batch, variant), the first row that fits; past
+// DX(log2N, type, largest n * batch, variant), type 0 FP32, 1 / 2 FP16 / BF16
+// tensor cores, 3 complex32; the first row that fits; past
 // the last one, variant 0 (FP32) or the first variant of the type.  A default
 // set by fft_set_default_variant (the autotuner's) goes before all of this.
 //
@@ -218,6 +230,11 @@
 // 2048 681 / 643; BF16 655 / 603, 643 / 600, 704 / 660, 665 / 632.  (Radix 16
 // first and last was faster still by 2-9% at 1024 and 2048, but rounds other
 // stages' operands to 16 bits.)
+//
+// complex32 (type 3), us, fixed stride / taken tiles: N = 4 2^24 26.2 / 23.8, 8
+// 2^27 179 / 163, 16 2^27 174 / 158, 32 2^27 165 / 160, 64 2^27 169 / 164, 128
+// 2^27 178 / 169, 256 2^27 181 / 169, 1024 2^27 218 / 213, 2048 2^27 240 / 232;
+// N = 2 (211 / 237) and N = 512 (208 / 208) keep the fixed stride.
 #define GBFFT_SIZE_DEFAULTS(DX) \
     DX(1, 0, 5 << 20, 4)        \
     DX(2, 0, 5 << 20, 6)        \
@@ -255,7 +272,24 @@
     DX(11, 1, 20 << 20, 4)      \
     DX(11, 1, INT64_MAX, 21)    \
     DX(11, 2, 20 << 20, 5)      \
-    DX(11, 2, INT64_MAX, 22)
+    DX(11, 2, INT64_MAX, 22)    \
+    DX(1, 3, 1 << 17, 3)        \
+    DX(2, 3, 12 << 20, 4)       \
+    DX(2, 3, INT64_MAX, 7)      \
+    DX(3, 3, INT64_MAX, 6)      \
+    DX(4, 3, INT64_MAX, 7)      \
+    DX(5, 3, INT64_MAX, 6)      \
+    DX(6, 3, 16 << 20, 1)       \
+    DX(6, 3, INT64_MAX, 7)      \
+    DX(7, 3, 14 << 20, 5)       \
+    DX(7, 3, INT64_MAX, 13)     \
+    DX(8, 3, 1 << 19, 18)       \
+    DX(8, 3, 12 << 20, 5)       \
+    DX(8, 3, INT64_MAX, 24)     \
+    DX(10, 3, 48 << 20, 8)      \
+    DX(10, 3, INT64_MAX, 19)    \
+    DX(11, 3, 20 << 20, 8)      \
+    DX(11, 3, INT64_MAX, 23)
 
 #define GBFFT_MIN_LOG2N 1
 #define GBFFT_MAX_LOG2N 11

@@ -18,7 +18,7 @@ from tests.helpers import FP32_TOL, c32_decode, c32_encode, c32_to, rel_l2_per_s
 from tests.test_bank_model import _rows, wavefronts
 
 PAIR_ROWS = [dict(L=r[0], variant=r[1], E=r[2], S=r[3], radix=[x for x in r[4:8] if x], D=r[9])
-             for r in _rows("GBFFT_C32_SCHEDULES", 11) if r[10] == 6]
+             for r in _rows("GBFFT_C32_SCHEDULES", 11) if r[10] & 7 == 6]
 IDS = [f"N{1 << r['L']}-v{r['variant']}" for r in PAIR_ROWS]
 # binary16 storage of every output component, plus the FP32 arithmetic
 C32_TOL = 2.0 ** -11 + FP32_TOL

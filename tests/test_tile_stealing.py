@@ -51,6 +51,40 @@ def test_every_tile_once(n, variant):
         ref.close()
 
 
+C32_ROWS = [(1 << r[0], r[1]) for r in _rows("GBFFT_C32_SCHEDULES", 11) if r[10] & 15 == 14] + \
+           [(1 << r[0], r[1]) for r in _rows("GBFFT_C32_SMALL_SCHEDULES", 5) if r[4] & 4]
+C32_FIXED = {1 << r[0]: r[1] for r in _rows("GBFFT_C32_SCHEDULES", 11) if r[10] in (0, 6)}
+
+
+@pytest.mark.parametrize("inverse", [False, True])
+@pytest.mark.parametrize("n,variant", C32_ROWS)
+def test_complex32_tiles_bit_for_bit(n, variant, inverse):
+    """Against a fixed-stride row of the same arithmetic (N <= 32: the direct
+    kernel splits the length, so there the results agree to one stored ulp)."""
+    probe = _plan(n, 1 << 22, variant)
+    resident, s = probe.info().grid, probe.info().signals_per_block
+    probe.close()
+    for batch in (1, s + 1, resident * s - 1, 2 * resident * s + 3, 5 * resident * s + s // 2):
+        g = torch.Generator(device="cuda").manual_seed(batch)
+        x = (torch.randn(batch, n, 2, generator=g, device="cuda") * 700).half()
+        e = torch.randint(-20, 20, (batch,), generator=g, device="cuda").to(torch.int8)
+        got = []
+        for v in (variant, C32_FIXED[n]):
+            y, f = torch.full_like(x, 3.0), torch.full_like(e, 77)
+            p = _plan(n, batch, v, inverse=inverse)
+            p.execute_c32(torch.view_as_complex(x), e, torch.view_as_complex(y), f)
+            assert p.error() == 0
+            p.close()
+            got.append((y, f))
+        if n > 32:
+            assert torch.equal(got[0][0].view(torch.int16), got[1][0].view(torch.int16))
+            assert torch.equal(got[0][1], got[1][1])
+        else:
+            d = [y.double() * torch.pow(2.0, f.double())[:, None, None] for y, f in got]
+            top = d[1].abs().amax(dim=(1, 2), keepdim=True)
+            assert float(((d[0] - d[1]).abs() / top).max()) <= 2.0 ** -10
+
+
 @pytest.mark.parametrize("n,variant", [(8, 0), (64, 0), (512, 0), (2048, 0), (2048, 22)])
 def test_launches_share_nothing_and_stay_in_order(n, variant):
     batch = (1 << 23) // n + 7
@@ -73,6 +107,22 @@ def test_launches_share_nothing_and_stay_in_order(n, variant):
     assert float(((a - x).norm(dim=1) / x.norm(dim=1)).max()) <= tol
     fwd.close()
     inv.close()
+
+
+@pytest.mark.parametrize("n,variant", [(64, 7), (256, 24), (2048, 23)])
+def test_a_stalled_complex32_grid_ends_after_one_wait(n, variant):
+    batch = (1 << 26) // n
+    x = torch.zeros(batch, n, 2, dtype=torch.float16, device="cuda")
+    e = torch.zeros(batch, dtype=torch.int8, device="cuda")
+    y, f = torch.full_like(x, 3.0), torch.full_like(e, 77)
+    plan = _plan(n, batch, variant, extra_flags=gb.FFT_FLAG_TEST_STALL)
+    plan.set_wait_limit(100_000_000)
+    t0 = time.perf_counter()
+    plan.execute_c32(torch.view_as_complex(x), e, torch.view_as_complex(y), f)
+    assert plan.error() == _abi.STATUS_CODE["FFT_ERR_TIMEOUT"]
+    assert time.perf_counter() - t0 < 3.0
+    assert torch.all(y == 3.0) and torch.all(f == 77)
+    plan.close()
 
 
 @pytest.mark.parametrize("n,variant", [(64, 0), (512, 0), (2048, 0), (256, 20), (1024, 18)])
