@@ -81,7 +81,11 @@ struct RCfg;
         using type = Cfg<L, E, S, R0, R1, R2, R3, 1, 0>; \
         static_assert(type::NT == 256, "ragged tiles use 256 threads"); \
     };
-// variant 0: E = 16 for N >= 32
+// variant 0: E = 16 for N >= 32.  Radix 16 first and last at N = 512 and 1024
+// (20000 signals of 2^4..2^11 in one launch 33.8 -> 32.9 us, all N = 512 30.5 ->
+// 28.9, all N = 1024 31.5 -> 30.2 against [8, 8, 8] and [8, 16, 8]); at N = 2048
+// [16, 8, 16] does not fit the producer variants' register cap without spills
+// (32.4 us against 32.3 for [8, 16, 16])
 GBFFT_RCFG(0, 1, 2, 256, 2, 0, 0, 0)
 GBFFT_RCFG(0, 2, 2, 128, 2, 2, 0, 0)
 GBFFT_RCFG(0, 3, 4, 128, 2, 4, 0, 0)
@@ -90,8 +94,8 @@ GBFFT_RCFG(0, 5, 16, 128, 8, 4, 0, 0)
 GBFFT_RCFG(0, 6, 16, 64, 8, 8, 0, 0)
 GBFFT_RCFG(0, 7, 16, 32, 8, 16, 0, 0)
 GBFFT_RCFG(0, 8, 16, 16, 16, 16, 0, 0)
-GBFFT_RCFG(0, 9, 16, 8, 8, 8, 8, 0)
-GBFFT_RCFG(0, 10, 16, 4, 8, 16, 8, 0)
+GBFFT_RCFG(0, 9, 16, 8, 16, 2, 16, 0)
+GBFFT_RCFG(0, 10, 16, 4, 16, 4, 16, 0)
 GBFFT_RCFG(0, 11, 16, 2, 8, 16, 16, 0)
 // variant 1: E = 8 for N >= 16
 GBFFT_RCFG(1, 1, 2, 256, 2, 0, 0, 0)
@@ -621,17 +625,22 @@ __device__ __forceinline__ void ragged_slot_body(const RaggedArgs& a) {
     }
     int it = blockIdx.x;
     if (it >= a.n_items) return;
-    RaggedItem w = a.items[it];
-    int64_t off = slot_offset_for<NTC>(a, w);
+    // of an item this thread keeps its signal's offset, and log2n, contig and
+    // count in one word (registers decide how many blocks fit)
+    auto fetch = [&](int i, int64_t& o) {
+        const RaggedItem x = a.items[i];
+        o = slot_offset_for<NTC>(a, x);
+        return (uint32_t)(x.log2n | x.contig << 8 | x.count << 16);
+    };
+    int64_t off = 0;
+    uint32_t meta = fetch(it, off);
     bool dead = false;
     for (int k = 0;; ++k) {
         const int nx = it + grid;
-        RaggedItem wn{};
+        uint32_t metan = 0;
         int64_t offn = 0;
-        if (nx < a.n_items) {  // the next item's descriptor and this thread's offset, ahead of time
-            wn = a.items[nx];
-            offn = slot_offset_for<NTC>(a, wn);
-        }
+        if (nx < a.n_items) metan = fetch(nx, offn);  // the next item's, ahead of time
+        const RaggedItem w = {(int)(meta & 255), (int)(meta >> 16), 0, (int)(meta >> 8 & 255), 0};
         const int slot = k % kSlots;
         if (!dead && !mbar_wait_bounded(&full[slot], (uint32_t)((k / kSlots) & 1), a.wait_ns)) {
             dead = true;
@@ -649,7 +658,7 @@ __device__ __forceinline__ void ragged_slot_body(const RaggedArgs& a) {
         }
         if (nx >= a.n_items) break;
         it = nx;
-        w = wn;
+        meta = metan;
         off = offn;
     }
 }
