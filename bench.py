@@ -618,7 +618,7 @@ def run_ours(args):
                "steps": e_steps, "step_ms": {"median": round(statistics.median(step_ms), 3),
                                              "mean": round(statistics.mean(step_ms), 3),
                                              "min": round(min(step_ms), 3), "max": round(max(step_ms), 3)},
-               "api": "fft_execute_host (pinned host buffers, 3-stream chunk pipeline)"}
+               "api": "fft_execute_host (pinned host buffers, one launch over mapped host memory)"}
         for p in hplans.values():
             p.close()
         del hx, hy

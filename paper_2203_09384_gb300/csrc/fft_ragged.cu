@@ -966,8 +966,7 @@ fft_status_t ragged_execute(RaggedState* st, const void* in, void* out, void* st
     args.out = static_cast<float2*>(out);
     void* kargs[] = {&args};
     if (launch_kernel(ragged_kernel(st->variant, st->inverse), (unsigned)st->grid,
-                      (unsigned)ragged_threads(st->variant), kargs, (size_t)st->smem, s,
-                      st->end - st->begin) != cudaSuccess) {
+                      (unsigned)ragged_threads(st->variant), kargs, (size_t)st->smem, s) != cudaSuccess) {
         cudaGetLastError();
         return FFT_ERR_CUDA;
     }

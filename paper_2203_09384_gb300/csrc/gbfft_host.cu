@@ -135,8 +135,7 @@ thread_local int t_plan_allocs = 0;
 }
 void begin_plan_allocs() { t_plan_allocs = 0; }
 cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, void** args, size_t smem,
-                          cudaStream_t stream, int64_t elems) {
-    if (elems < kPdlMinElems) return cudaLaunchKernel(kernel, dim3(grid), dim3(block), args, smem, stream);
+                          cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -222,12 +221,12 @@ fft_status_t launch_plain(gbfft_plan* p, const gbfft_plan::Launch& l, const floa
     if (e->kind == KernelKind::Small && !e->steal) {
         void* args[] = {&in2, &out2, &batch, &scale};
         ce = gbfft::launch_kernel(l.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
-                                  (size_t)e->smem_bytes, stream, batch * p->n);
+                                  (size_t)e->smem_bytes, stream);
     } else {
         int stall = (p->flags & FFT_FLAG_TEST_STALL) ? 1 : 0;
         void* args[] = {&in2, &out2, &batch, &tw, &scale, &err, &wait_ns, &stall};
         ce = gbfft::launch_kernel(l.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
-                                  (size_t)e->smem_bytes, stream, batch * p->n);
+                                  (size_t)e->smem_bytes, stream);
     }
     if (ce != cudaSuccess) {
         cudaGetLastError();
@@ -620,7 +619,7 @@ fft_status_t fft_execute_c32(fft_plan_t p, const void* in, const int8_t* in_exp,
     void* args[] = {&in2, &in_exp, &out2, &out_exp, &batch, &tw, &scale, &err, &wait_ns, &stall};
     const int64_t grid = e->steal ? (batch + e->signals_per_block - 1) / e->signals_per_block : p->grid;
     if (gbfft::launch_kernel(p->dev.kernel, (unsigned)grid, (unsigned)e->threads_per_block, args,
-                             (size_t)e->smem_bytes, (cudaStream_t)stream, batch * p->n) != cudaSuccess) {
+                             (size_t)e->smem_bytes, (cudaStream_t)stream) != cudaSuccess) {
         cudaGetLastError();
         return FFT_ERR_CUDA;
     }
