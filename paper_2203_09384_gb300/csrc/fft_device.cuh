@@ -15,12 +15,12 @@
 // and the last stage leaves the result in natural order (no bit reversal).
 //
 // GB300 mapping: each thread keeps E complex elements in registers and runs
-// E/R butterflies per stage.  Stage 0 reads straight from HBM and the last
-// stage writes straight to HBM, with 128-bit accesses whenever a thread owns
-// two neighbouring butterflies; stages exchange through shared memory with an
-// XOR swizzle (conflict free for N = 128, 256, 1024, 2048; 1.25x the minimum
-// wavefronts at N = 512 and 1.5x at N = 32 and 64, where HBM still bounds the
-// kernel).  A persistent grid-stride loop walks tiles of S signals.
+// E/R butterflies per stage.  Input comes straight from HBM or through a ring
+// of bulk copies; the last stage writes straight to HBM, with 128-bit accesses
+// whenever a thread owns two neighbouring butterflies; stages exchange through
+// shared memory with an XOR swizzle (swz8 below).  Tiles of S signals are
+// walked with the grid's stride or, in large calls, taken from blocks that
+// have not started (TileTaker).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -245,8 +245,8 @@ __device__ __forceinline__ void st_stream4v(float4* p, float4 a) {
 // (signals starting every 2 or 4 rows) take 1.5x the conflict-free
 // wavefronts; with row >> 2 folded in none conflicts.  The other lengths keep
 // the cheaper form (measured, the folded one cost the N = 2048 ring kernel
-// 1.4 points); their defaults model at 1.0x, except N = 512 (1.25x) and the
-// exchanges of the N = 128 padded in-ring default (1.33x).
+// 1.4 points); the FP32 defaults model at 1.0x, except the padded in-ring
+// kernel of N = 128 (1.33x) and the mid-size kernel of N = 64 (1.5x).
 // tests/test_bank_model.py replays every schedule's exchanges under it and
 // counts the wavefronts (64-bit accesses resolve per half-warp), in agreement
 // with ncu.
