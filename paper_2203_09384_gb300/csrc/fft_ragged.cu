@@ -17,7 +17,7 @@
 // flight.  Variants 5..9 run set 0 in ring slots that a producer warp fills
 // (exchanges inside the slot): 5 with 256 compute threads and 2 slots, 6 with
 // 128 compute threads and 2 slots, 7 with 128 and 3 slots, 8 as 6 with
-// registers capped at 80, 9 (the default) the kernel of 8 with the lengths up
+// registers capped at 96, 9 (the default) the kernel of 8 with the lengths up
 // to 128 first in the work list.
 // A tile whose signals lie back to back (runs of one length in the input)
 // is marked at plan time: its threads compute their offsets instead of
@@ -83,9 +83,9 @@ struct RCfg;
     };
 // variant 0: E = 16 for N >= 32.  Radix 16 first and last at N = 512 and 1024
 // (20000 signals of 2^4..2^11 in one launch 33.8 -> 32.9 us, all N = 512 30.5 ->
-// 28.9, all N = 1024 31.5 -> 30.2 against [8, 8, 8] and [8, 16, 8]); at N = 2048
-// [16, 8, 16] does not fit the producer variants' register cap without spills
-// (32.4 us against 32.3 for [8, 16, 16])
+// 28.9, all N = 1024 31.5 -> 30.2 against [8, 8, 8] and [8, 16, 8]); the same
+// at N = 2048 (all N = 2048 32.3 -> 30.5 against [8, 16, 16]), which needs the
+// compute threads free of descriptors (SlotInfo) to fit 96 registers
 GBFFT_RCFG(0, 1, 2, 256, 2, 0, 0, 0)
 GBFFT_RCFG(0, 2, 2, 128, 2, 2, 0, 0)
 GBFFT_RCFG(0, 3, 4, 128, 2, 4, 0, 0)
@@ -96,7 +96,7 @@ GBFFT_RCFG(0, 7, 16, 32, 8, 16, 0, 0)
 GBFFT_RCFG(0, 8, 16, 16, 16, 16, 0, 0)
 GBFFT_RCFG(0, 9, 16, 8, 16, 2, 16, 0)
 GBFFT_RCFG(0, 10, 16, 4, 16, 4, 16, 0)
-GBFFT_RCFG(0, 11, 16, 2, 8, 16, 16, 0)
+GBFFT_RCFG(0, 11, 16, 2, 16, 8, 16, 0)
 // variant 1: E = 8 for N >= 16
 GBFFT_RCFG(1, 1, 2, 256, 2, 0, 0, 0)
 GBFFT_RCFG(1, 2, 2, 128, 2, 2, 0, 0)
@@ -115,7 +115,7 @@ GBFFT_RCFG(1, 11, 8, 1, 4, 8, 8, 8)
 // schedule set 1 shapes fed by a bulk-copy (TMA) prefetch ring; variants 5..8:
 // set 0 shapes in ring slots filled by a producer warp (5: 256 compute threads
 // and 2 slots; 6 / 7: 128 compute threads, half the signals per tile, 2 / 3
-// slots, 4 resident blocks per SM; 8: as 6 with registers capped at 80;
+// slots, 4 resident blocks per SM; 8: as 6 with registers capped at 96;
 // 9: as 8, short lengths first in the work list)
 constexpr int kRaggedVariants = 10;
 constexpr int kRingVariant = 4;
@@ -152,6 +152,23 @@ struct SlotCfg {
     using type = Cfg<L, B::E, B::S * NTC / kRaggedThreads, B::radix(0), B::radix(1), B::radix(2), B::radix(3), 2, 2,
                      0, -1, CH>;
     static_assert(type::NT == NTC, "one tile per compute group");
+};
+// expect bytes on a barrier, its arrival following separately
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
+// What the producer warp tells the compute threads of the item in a slot: its
+// length, count and contig (one word) and the element offsets of its signals
+// (of a back-to-back tile only the first).  They read it from shared memory
+// behind the slot's `full` barrier.  When each of them loaded and kept the next
+// item's descriptor and offset itself, N = 2048 spilled with radices
+// [16, 8, 16]; a call of 20000 signals of 2^4..2^11 took 33.0 us, now 31.8
+// (256..2048 28.4 -> 27.2, all N = 2048 32.4 -> 30.5, 2..32 11.95 -> 11.8).
+template <int NTC>
+struct SlotInfo {
+    int64_t off[NTC];  // at most one signal per thread
+    uint32_t meta;     // log2n | contig << 8 | count << 16
 };
 template <int NTC, int MINB>
 struct SlotShape {
@@ -498,10 +515,13 @@ __device__ __forceinline__ void slot_gather0(float2 (&v)[C::E], const float2* ti
 
 template <class C, bool INV>
 __device__ __forceinline__ void slot_tile(const RaggedArgs& a, const RaggedItem& w, float2* slot, uint64_t* empty,
-                                          int64_t off, bool dead) {
+                                          const int64_t* offs, bool dead) {
     static_assert(C::S * C::N <= C::NT * 16, "a tile must fit a ring slot");
     static_assert(C::S * (C::N + slot_pad_of<C>()) <= C::NT * 17, "a padded tile must fit a ring slot");
-    const int tid = threadIdx.x;
+    // N = 2048 reads its thread index anew for each item: addresses made from
+    // threadIdx are hoisted out of the item loop, and with them it spilled
+    int tid = threadIdx.x;
+    if constexpr (C::LOG2N == 11) asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
     const int sl = tid / C::T;
     const int t = tid % C::T;
     const bool active = sl < w.count && !dead;
@@ -519,36 +539,29 @@ __device__ __forceinline__ void slot_tile(const RaggedArgs& a, const RaggedItem&
         if (padded) asm volatile("bar.sync %0, %1;" ::"n"(bar_base<C::NT, 2 * C::NT>()), "n"(C::NT) : "memory");
     }
     slot_stages<C, 1>(v, slot, sl * C::N, t, tw, tc);
+    const int64_t off = offs[w.contig ? 0 : sl] + (w.contig ? (int64_t)sl << C::LOG2N : 0);
     // this thread is done with the slot: order its shared-memory accesses
     // before the producer's next copy into it; once the whole warp is, one
-    // lane releases the slot for the warp (the barrier counts warps)
+    // lane releases the slot for the warp (the barrier counts warps).  A warp
+    // that gave up waiting releases nothing: its arrival could stand in for
+    // that of a warp still reading the slot and its SlotInfo
     fence_proxy_async_smem();
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
+    if ((threadIdx.x & 31) == 0 && !dead) mbar_arrive(empty);
     store_last<C, INV>(v, a.out + off, t, active, scale);
 }
 
-template <int NTC>
-__device__ __forceinline__ int64_t slot_offset_for(const RaggedArgs& a, const RaggedItem& w) {
-    switch (w.log2n) {
-#define GBFFT_SOFF(L) \
-    case L: return ragged_offset<typename SlotCfg<NTC, L>::type>(a, w);
-        GBFFT_SOFF(1) GBFFT_SOFF(2) GBFFT_SOFF(3) GBFFT_SOFF(4) GBFFT_SOFF(5) GBFFT_SOFF(6)
-        GBFFT_SOFF(7) GBFFT_SOFF(8) GBFFT_SOFF(9) GBFFT_SOFF(10) GBFFT_SOFF(11)
-#undef GBFFT_SOFF
-        default: return 0;
-    }
-}
-
 // The producer warp.  Lane 0 sets each fill's byte count; every lane copies
-// signals lane, lane + 32, ...  The next item's descriptor is loaded before
-// the wait for a free slot, so its latency hides behind that wait, and a
-// tile's first signal comes with its own offset (RaggedItem::off0), so a
-// single-signal tile costs one global load before its copy, not two.  Before
-// it exits, lane 0 waits (bounded) for the copies it issued last, so none
+// signals lane, lane + 32, ..., then writes their offsets to the slot's
+// SlotInfo, and lane 0's arrival on `full` ends the fill.  The next item's
+// descriptor is loaded before the wait for a free slot, and the offsets of a
+// tile of scattered signals after the copies of the item before, so that their
+// latency hides behind that wait.  A back-to-back tile's first signal comes
+// with its own offset (RaggedItem::off0).  Before it exits, lane 0 waits (bounded) for the copies it issued last, so none
 // lands after the block is gone even when the compute threads gave up.
 template <int NTC, int SLOTS, int MINB>
-__device__ __forceinline__ void slot_produce(const RaggedArgs& a, float2* ring, uint64_t* full, uint64_t* empty) {
+__device__ __forceinline__ void slot_produce(const RaggedArgs& a, float2* ring, uint64_t* full, uint64_t* empty,
+                                             SlotInfo<NTC>* info) {
     constexpr int kSlots = SLOTS;
     constexpr int kSlotTile = SlotShape<NTC, MINB>::kTile;
     const int lane = threadIdx.x & 31;
@@ -559,6 +572,15 @@ __device__ __forceinline__ void slot_produce(const RaggedArgs& a, float2* ring, 
     int it = blockIdx.x;
     if (it >= a.n_items) return;
     RaggedItem w = a.items[it];
+    constexpr int kOwn = NTC / 32;  // signals per lane at most
+    int64_t o[kOwn];
+    auto load_offsets = [&](const RaggedItem& x) {
+        if (x.contig) return;
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i)
+            if (lane + 32 * i < x.count) o[i] = a.sig_off[x.first + lane + 32 * i];
+    };
+    load_offsets(w);
     for (int k = 0;; ++k) {
         const int slot = k % kSlots;
         const int nx = it + (int)gridDim.x;
@@ -576,24 +598,41 @@ __device__ __forceinline__ void slot_produce(const RaggedArgs& a, float2* ring, 
         const int n = 1 << w.log2n;
         float2* dst = ring + slot * kSlotTile;
         if (lane == 0) {
-            mbar_arrive_expect_tx(&full[slot], (uint32_t)(w.count * n * 8));
+            mbar_expect_tx(&full[slot], (uint32_t)(w.count * n * 8));
             inflight.issued(slot, (uint32_t)((k / kSlots) & 1));
         }
-        __syncwarp();
+        __syncwarp();  // the bytes are expected, and lane 0's wait for the slot's last readers covers every lane
         if (w.contig && n < kSpanChunk) {  // one span of short signals: copies of kSpanChunk elements
             const int total = w.count * n;
             for (int j = lane * kSpanChunk; j < total; j += 32 * kSpanChunk)
                 bulk_copy_g2s(dst + j, a.in + w.off0 + j, (uint32_t)(min(kSpanChunk, total - j) * 8), &full[slot]);
+        } else if (w.contig) {
+            // the offsets could be computed, but copies issued that much sooner
+            // crowd out the stores of the item before (all N = 256 29.4 us, so 27.5)
+            for (int j = lane; j < w.count; j += 32)
+                bulk_copy_g2s(dst + j * n, a.in + (j == 0 ? w.off0 : a.sig_off[w.first + j]), (uint32_t)(n * 8),
+                              &full[slot]);
         } else {
             // scattered signals, one copy each, every n + pad elements (slot_pad)
-            const int pitch = n + (w.count > 1 ? slot_pad<NTC>(w.log2n) : 0);
-            for (int j = lane; j < w.count; j += 32)
-                bulk_copy_g2s(dst + j * pitch, a.in + (j == 0 ? w.off0 : a.sig_off[w.first + j]), (uint32_t)(n * 8),
-                              &full[slot]);
+            const int pitch = n + slot_pad<NTC>(w.log2n);
+#pragma unroll
+            for (int i = 0; i < kOwn; ++i) {
+                const int j = lane + 32 * i;
+                if (j >= w.count) break;
+                bulk_copy_g2s(dst + j * pitch, a.in + o[i], (uint32_t)(n * 8), &full[slot]);
+                info[slot].off[j] = o[i];
+            }
         }
+        if (lane == 0) {
+            if (w.contig) info[slot].off[0] = w.off0;
+            info[slot].meta = (uint32_t)(w.log2n | w.contig << 8 | w.count << 16);
+        }
+        __syncwarp();  // lane 0's arrival releases what every lane wrote
+        if (lane == 0) mbar_arrive(&full[slot]);
         if (nx >= a.n_items) break;
         it = nx;
         w = wn;
+        load_offsets(w);
     }
     if (lane == 0) inflight.drain(full, a.wait_ns);
 }
@@ -608,8 +647,8 @@ __device__ __forceinline__ void ragged_slot_body(const RaggedArgs& a) {
     float2* ring = smem;  // kSlots slots of kSlotTile elements
     uint64_t* full = reinterpret_cast<uint64_t*>(ring + kSlots * kSlotTile);
     uint64_t* empty = full + kSlots;
+    SlotInfo<NTC>* info = reinterpret_cast<SlotInfo<NTC>*>(empty + kSlots);
     const int tid = threadIdx.x;
-    const int grid = (int)gridDim.x;
     dbg_set_err(a.err);
     if (tid == 0) {
         for (int d = 0; d < kSlots; ++d) {
@@ -620,46 +659,35 @@ __device__ __forceinline__ void ragged_slot_body(const RaggedArgs& a) {
     }
     __syncthreads();  // the last barrier of all NTC + 32 threads
     if (tid >= NTC) {
-        slot_produce<NTC, SLOTS, MINB>(a, ring, full, empty);
+        slot_produce<NTC, SLOTS, MINB>(a, ring, full, empty, info);
         return;
     }
-    int it = blockIdx.x;
-    if (it >= a.n_items) return;
-    // of an item this thread keeps its signal's offset, and log2n, contig and
-    // count in one word (registers decide how many blocks fit)
-    auto fetch = [&](int i, int64_t& o) {
-        const RaggedItem x = a.items[i];
-        o = slot_offset_for<NTC>(a, x);
-        return (uint32_t)(x.log2n | x.contig << 8 | x.count << 16);
-    };
-    int64_t off = 0;
-    uint32_t meta = fetch(it, off);
     bool dead = false;
-    for (int k = 0;; ++k) {
-        const int nx = it + grid;
-        uint32_t metan = 0;
-        int64_t offn = 0;
-        if (nx < a.n_items) metan = fetch(nx, offn);  // the next item's, ahead of time
-        const RaggedItem w = {(int)(meta & 255), (int)(meta >> 16), 0, (int)(meta >> 8 & 255), 0};
+    int k = 0;
+    for (int it = blockIdx.x; it < a.n_items; it += (int)gridDim.x, ++k) {
         const int slot = k % kSlots;
         if (!dead && !mbar_wait_bounded(&full[slot], (uint32_t)((k / kSlots) & 1), a.wait_ns)) {
             dead = true;
             atomicCAS(a.err, 0, kErrTimeout);
         }
+        RaggedItem w;
+        if (!dead) {
+            const uint32_t meta = info[slot].meta;
+            w = {(int)(meta & 255), (int)(meta >> 16), 0, (int)(meta >> 8 & 255), 0};
+        } else {
+            w = a.items[it];  // the slot holds nothing; the shape decides the barriers to take part in
+        }
         switch (w.log2n) {
 #define GBFFT_SCASE(L)                                                                                       \
     case L:                                                                                                  \
-        slot_tile<typename SlotCfg<NTC, L, CH>::type, INV>(a, w, ring + slot * kSlotTile, &empty[slot], off, dead); \
+        slot_tile<typename SlotCfg<NTC, L, CH>::type, INV>(a, w, ring + slot * kSlotTile, &empty[slot],      \
+                                                           info[slot].off, dead);                            \
         break;
             GBFFT_SCASE(1) GBFFT_SCASE(2) GBFFT_SCASE(3) GBFFT_SCASE(4) GBFFT_SCASE(5) GBFFT_SCASE(6)
             GBFFT_SCASE(7) GBFFT_SCASE(8) GBFFT_SCASE(9) GBFFT_SCASE(10) GBFFT_SCASE(11)
 #undef GBFFT_SCASE
             default: break;
         }
-        if (nx >= a.n_items) break;
-        it = nx;
-        meta = metan;
-        off = offn;
     }
 }
 
@@ -673,10 +701,9 @@ __global__ void __launch_bounds__(SlotShape<NTC, MINB>::kThreads, SlotShape<NTC,
 }
 
 // Registers capped at REGS per thread directly.  (Registers are allocated per
-// SM sub-partition, 4 x 16K, a warp at a time: at 80 registers 4 blocks of 5
-// warps fit per SM, 5 would need 72 or fewer.  Measured: a 72-register form,
-// with the next item loaded late to avoid spills, ran 5 blocks per SM and was
-// no faster.)
+// SM sub-partition, 4 x 16K, a warp at a time: at 96 registers 4 blocks of 5
+// warps fit per SM; 5 would need 72 and 6 would need 64, and were slower:
+// 20000 signals of 2^4..2^11 36.1 and 36.3 us, against 32.5 at 80 and 96.)
 template <int NTC, int SLOTS, int REGS, int CH, bool INV>
 __global__ void __maxnreg__(REGS) fft_ragged_slot_kernel_capped(RaggedArgs a) {
     pdl_enter();
@@ -779,8 +806,8 @@ const void* ragged_kernel(int v, bool inv) {
                        : reinterpret_cast<const void*>(&fft_ragged_slot_kernel<128, 3, 4, false>);
         case 8:
         case 9:
-            return inv ? reinterpret_cast<const void*>(&fft_ragged_slot_kernel_capped<128, 2, 80, 0, true>)
-                       : reinterpret_cast<const void*>(&fft_ragged_slot_kernel_capped<128, 2, 80, 0, false>);
+            return inv ? reinterpret_cast<const void*>(&fft_ragged_slot_kernel_capped<128, 2, 96, 0, true>)
+                       : reinterpret_cast<const void*>(&fft_ragged_slot_kernel_capped<128, 2, 96, 0, false>);
         default:
             return inv ? reinterpret_cast<const void*>(&fft_ragged_ring_kernel<true>)
                        : reinterpret_cast<const void*>(&fft_ragged_ring_kernel<false>);
@@ -788,7 +815,10 @@ const void* ragged_kernel(int v, bool inv) {
 }
 int ragged_smem(int v) {
     if (v == kRingVariant) return 4 * kRingTile * (int)sizeof(float2) + 16;
-    if (is_producer_variant(v)) return producer_slots(v) * producer_group(v) * 17 * (int)sizeof(float2) + 2 * producer_slots(v) * 8;
+    if (is_producer_variant(v)) {
+        const int info = producer_group(v) == 256 ? sizeof(SlotInfo<256>) : sizeof(SlotInfo<128>);
+        return producer_slots(v) * (producer_group(v) * 17 * (int)sizeof(float2) + 2 * 8 + info);
+    }
     return schedule_set(v) == 0 ? ragged_smem_bytes<0>() : ragged_smem_bytes<1>();
 }
 
