@@ -5,7 +5,7 @@
 // tiles of S_N signals (the same per-length schedules as the uniform path,
 // re-shaped so that every length runs in a 256-thread block), and the tiles
 // become a device work list ordered from the longest length down (variant 9:
-// the lengths up to 128 first, then the rest longest first).
+// the lengths up to 128 first, then the rest longest first; long lists ascend).
 //
 // Ten variants are compiled.  Bit 0 of variants 0..3 picks the schedule
 // set: set 0 keeps 16 complex elements per thread for N >= 32 (fewest
@@ -18,7 +18,7 @@
 // (exchanges inside the slot): 5 with 256 compute threads and 2 slots, 6 with
 // 128 compute threads and 2 slots, 7 with 128 and 3 slots, 8 as 6 with
 // registers capped at 96, 9 (the default) the kernel of 8 with the lengths up
-// to 128 first in the work list.
+// to 128 first in the work list, or all lengths ascending in a long list.
 // A tile whose signals lie back to back (runs of one length in the input)
 // is marked at plan time: its threads compute their offsets instead of
 // loading them, and the bulk-copy variants fetch a tile of short signals in
@@ -123,6 +123,14 @@ constexpr int kFirstProducerVariant = 5;
 constexpr int kDefaultRaggedVariant = 9;  // measured fastest on the mixed-length workload
 constexpr int kShortFirstVariant = 9;     // variant 8's kernel, short lengths first in the work list
 constexpr int kShortMaxLog2n = 7;  // measured: up to 128 first beats up to 32 or 64 on the mix
+// Items a block from which variant 9's list ascends through all lengths.
+// Signals of 2^4..2^11, 128 at most first / all ascending, us: 5000 (2.1 items
+// a block) 11.1 / 12.4, 10000 (4.1) 18.6 / 18.8, 13000 (5.3) 22.4 / 22.9, 15000
+// (6.2) 25.4 / 25.0, 18000 (7.4) 29.6 / 28.4, 20000 31.9 / 31.0, 30000 46.3 / 42.7,
+// 40000 59.2 / 54.9; 256..2048, 9000 (6.9) 27.3 / 25.6.  Blocks keep to one
+// length's code longer; but the last items are the longest lengths' and cost
+// a short list more.  (Items by address instead, lengths mixed: 20000 42.5 us.)
+constexpr int64_t kAscendRounds = 6;
 // the variant ragged plans use when the caller names none (process-wide; the
 // autotuner's cached choice is applied through fft_set_default_ragged_variant)
 std::atomic<int> g_default_ragged_variant{kDefaultRaggedVariant};
@@ -877,18 +885,40 @@ fft_status_t ragged_create(const int64_t* offsets, int64_t count, int direction,
     st->begin = count > 0 ? offsets[0] : 0;
     st->end = count > 0 ? offsets[count] : 0;
 
-    // work list and the bucketed offsets.  Longest length first, so that the
+    // launch shape: persistent, every SM filled
+    const void* k = ragged_kernel(variant, st->inverse);
+    st->smem = ragged_smem(variant);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        (st->smem > 48 * 1024 &&
+         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, st->smem) != cudaSuccess) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, ragged_threads(variant), st->smem) != cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        delete st;
+        return FFT_ERR_CUDA;
+    }
+    const int64_t resident = (int64_t)sms * per_sm;
+
+    // Work list and the bucketed offsets.  Longest length first, so that the
     // last items, which run while the machine drains, are short; variant 9
     // takes the lengths up to 128 (tiles of many short signals, one bulk copy
     // each) first instead, then the rest longest first, so the final items
-    // are the N = 256 tiles (8 signals each).  (The named barriers of the producer
-    // variants allow any order, see slot_sync.)
-    std::vector<int> order;
+    // are the N = 256 tiles (8 signals each), and in work lists of kAscendRounds
+    // items a block or more every length in ascending order.  (The named
+    // barriers of the producer variants allow any order, see slot_sync.)
     const bool short_first = variant >= kShortFirstVariant;
-    if (short_first)
-        for (int L = GBFFT_MIN_LOG2N; L <= kShortMaxLog2n; ++L) order.push_back(L);
+    int64_t n_items = 0;
+    for (int L = GBFFT_MIN_LOG2N; L <= GBFFT_MAX_LOG2N; ++L) {
+        const int64_t S = signals_per_tile(variant, L);
+        if (S > 0) n_items += ((int64_t)buckets[L].size() + S - 1) / S;
+    }
+    const int ascending = !short_first ? 0 : n_items >= kAscendRounds * resident ? GBFFT_MAX_LOG2N : kShortMaxLog2n;
+    std::vector<int> order;
+    for (int L = GBFFT_MIN_LOG2N; L <= ascending; ++L) order.push_back(L);
     for (int L = GBFFT_MAX_LOG2N; L >= GBFFT_MIN_LOG2N; --L)
-        if (!short_first || L > kShortMaxLog2n) order.push_back(L);
+        if (L > ascending) order.push_back(L);
     std::vector<RaggedItem> items;
     std::vector<int64_t> sig;
     sig.reserve((size_t)count);
@@ -954,22 +984,6 @@ fft_status_t ragged_create(const int64_t* offsets, int64_t count, int direction,
     st->args.wait_ns = 4000000000ull;
     st->args.stall = (flags & FFT_FLAG_TEST_STALL) ? 1 : 0;
 
-    // launch shape: persistent, every SM filled
-    const void* k = ragged_kernel(variant, st->inverse);
-    st->smem = ragged_smem(variant);
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        (st->smem > 48 * 1024 &&
-         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, st->smem) != cudaSuccess) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, ragged_threads(variant), st->smem) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        cudaFree(st->dmem);
-        delete st;
-        return FFT_ERR_CUDA;
-    }
-    const int64_t resident = (int64_t)sms * per_sm;
     st->grid = st->n_items < resident ? st->n_items : resident;
     if (st->grid < 1) st->grid = 1;
     *out = st;
