@@ -131,6 +131,11 @@ constexpr int kShortMaxLog2n = 7;  // measured: up to 128 first beats up to 32 o
 // length's code longer; but the last items are the longest lengths' and cost
 // a short list more.  (Items by address instead, lengths mixed: 20000 42.5 us.)
 constexpr int64_t kAscendRounds = 6;
+// Blocks from which a launch may overlap the kernel before it.  Calls chained
+// in one graph, plain / overlapped, us: 200 signals of 2^4..2^11 (50 blocks)
+// 3.30 / 3.46, 300 (75) 3.71 / 3.64, 500 4.54 / 4.47, 800 4.99 / 4.45, 2000
+// 6.68 / 5.92.  One item a block leaves nothing to overlap but the ramp.
+constexpr int64_t kProgrammaticGrid = 64;
 // the variant ragged plans use when the caller names none (process-wide; the
 // autotuner's cached choice is applied through fft_set_default_ragged_variant)
 std::atomic<int> g_default_ragged_variant{kDefaultRaggedVariant};
@@ -1010,7 +1015,8 @@ fft_status_t ragged_execute(RaggedState* st, const void* in, void* out, void* st
     args.out = static_cast<float2*>(out);
     void* kargs[] = {&args};
     if (launch_kernel(ragged_kernel(st->variant, st->inverse), (unsigned)st->grid,
-                      (unsigned)ragged_threads(st->variant), kargs, (size_t)st->smem, s) != cudaSuccess) {
+                      (unsigned)ragged_threads(st->variant), kargs, (size_t)st->smem, s,
+                      st->grid >= kProgrammaticGrid) != cudaSuccess) {
         cudaGetLastError();
         return FFT_ERR_CUDA;
     }

@@ -135,7 +135,7 @@ thread_local int t_plan_allocs = 0;
 }
 void begin_plan_allocs() { t_plan_allocs = 0; }
 cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, void** args, size_t smem,
-                          cudaStream_t stream) {
+                          cudaStream_t stream, bool programmatic) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -145,7 +145,7 @@ cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, voi
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = programmatic ? 1 : 0;
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
