@@ -46,9 +46,12 @@ def _cuda_device(device) -> torch.device:
     return d if d.index is not None else torch.device("cuda", torch.cuda.current_device())
 
 
-def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_least: bool = False) -> None:
+def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_least: bool = False,
+                  output: bool = False) -> None:
     """A buffer handed to the C-ABI as a bare pointer: the library cannot see
-    its size, dtype or device, so they are checked here before the launch."""
+    its size, dtype or device, so they are checked here before the launch.  An
+    output must not be a lazily conjugated view, which would read back as the
+    conjugate of what is stored."""
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
@@ -57,6 +60,18 @@ def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_leas
         raise ValueError(f"{name} is on {t.device}, expected {device}")
     if (t.numel() < numel) if at_least else (t.numel() != numel):
         raise ValueError(f"{name} has {t.numel()} elements, needs {'at least ' if at_least else ''}{numel}")
+    if output and t.is_conj():
+        raise ValueError(f"{name} must not be a lazily conjugated view")
+
+
+def _stored(t: torch.Tensor, stream=None) -> torch.Tensor:
+    """t with its values as they stand in memory: x.conj() is a view with a
+    flag, which is contiguous but keeps x's storage.  The copy is made on
+    `stream`, where the transform that reads it runs."""
+    if not t.is_conj():
+        return t
+    with torch.cuda.stream(stream):
+        return t.resolve_conj()
 
 
 # The two queries every call needs, without the wrappers' device objects,
@@ -109,11 +124,12 @@ class Plan:
         return fft_plan_get_info(self.handle)
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
+        x = _stored(x, stream)
         _check_buffer(x, "x", torch.complex64, self.device, self.n * self.batch)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex64, self.device, self.n * self.batch)
+            _check_buffer(out, "out", torch.complex64, self.device, self.n * self.batch, output=True)
         _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
@@ -122,12 +138,13 @@ class Plan:
         """complex32 storage (plan dtype "c32"): x is a torch.complex32 CUDA
         tensor, x_exp an int8 tensor of one exponent per signal (value =
         stored * 2^exp).  Returns (out, out_exp) in the same representation."""
+        x = _stored(x, stream)
         _check_buffer(x, "x", torch.complex32, self.device, self.n * self.batch)
         _check_buffer(x_exp, "x_exp", torch.int8, self.device, self.batch)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex32, self.device, self.n * self.batch)
+            _check_buffer(out, "out", torch.complex32, self.device, self.n * self.batch, output=True)
         if out_exp is None:
             out_exp = torch.empty(self.batch, dtype=torch.int8, device=x.device)
         else:
@@ -144,7 +161,8 @@ class Plan:
         if out is None:
             out = torch.empty(x.shape, dtype=x.dtype, pin_memory=x.is_pinned())
         else:
-            _check_buffer(out, "out", torch.complex64, cpu, self.n * self.batch)
+            _check_buffer(out, "out", torch.complex64, cpu, self.n * self.batch, output=True)
+        x = x.resolve_conj()  # a host copy, kept until the stream has been waited for below
         with torch.cuda.device(self.device):
             s = stream if stream is not None else torch.cuda.current_stream(self.device)
             fft_execute_host(self.handle, x.data_ptr(), out.data_ptr(), s.cuda_stream)
@@ -200,11 +218,12 @@ class RaggedPlan:
         return fft_plan_get_info(self.handle)
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
+        x = _stored(x, stream)
         _check_buffer(x, "x", torch.complex64, self.device, self.total, at_least=True)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex64, self.device, self.total, at_least=True)
+            _check_buffer(out, "out", torch.complex64, self.device, self.total, at_least=True, output=True)
         _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
@@ -288,7 +307,7 @@ def _run(x: torch.Tensor, inverse: bool, normalized: bool = True, dtype: str = "
     if not x.is_cuda:
         raise TypeError("gbfft works on CUDA tensors")
     n = x.shape[-1]
-    x = x.contiguous()
+    x = _stored(x.contiguous())
     batch = x.numel() // n if n > 0 else 0
     plan = get_plan(n, batch, inverse, normalized, x.device, dtype, scale_forward)
     out = torch.empty_like(x)
