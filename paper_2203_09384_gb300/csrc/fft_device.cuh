@@ -566,6 +566,9 @@ struct Cfg {
     __host__ __device__ static constexpr bool tc_stage(int s) {
         return TC != 0 && E == 16 && radix(s) == 16 && (!kTcLastOnly || s == kLast16);
     }
+    // stage 0 holds steps that a whole warp or block takes together: the MMA's
+    // barriers and TMEM accesses, or the reduction of the signal's maximum
+    static constexpr bool kStage0Together = kTcSignalScale || tc_stage(0);
     // Ns of stage s: product of the radices before it
     __host__ __device__ static constexpr int ns(int s) {
         int p = 1;
@@ -1440,7 +1443,11 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         if constexpr (C::kAInRing) tc.a = reinterpret_cast<unsigned char*>(b);
         const int64_t sig = tile * C::S + sl;
         float2 v[C::E];
-        if (!C::kSteal || tile >= 0) {
+        // threads with no tile (the end, or their own wait gave up) skip stage 0;
+        // where it is taken together none does, since other threads of the warp
+        // may have seen their wait succeed: once per block it then transforms
+        // what the slot holds, for nothing
+        if (!C::kSteal || C::kStage0Together || tile >= 0) {
             gather_tile<C, INV>(v, b, sl * (C::N + C::kSlotPad), t);
             tc_norm_begin<C>(v, tc);
             twist_and_dft<C, 0>(v, t, tw, tc);
