@@ -616,28 +616,27 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
                 atomicCAS(err, 0, kErrTimeout);
             }
         }
-        if constexpr (C::kSteal) {
-            tile = dead ? -1 : *slot_tile;
-            // every thread leaves in the same iteration, also when one gave up
-            if (tile < 0) {
-                __syncthreads_or(dead);
-                break;
-            }
-        }
+        if constexpr (C::kSteal) tile = dead ? -1 : *slot_tile;
         const int64_t sig = tile * C::S + 2 * pr;
-        const bool in_a = sig < batch, in_b = sig + 1 < batch;
-        const int ea = in_a ? (int)in_exp[sig] : 0, eb = in_b ? (int)in_exp[sig + 1] : 0;
-        const uint32_t* src =
-            reinterpret_cast<const uint32_t*>(base8 + C::kExchangeBytes + slot * C::kSlotBytes) + 2 * pr * C::N;
+        bool in_a = false, in_b = false;
+        int ea = 0, eb = 0;
         C2 v[C::E];
-        pair_load<C, INV>(v, src, t);
-        pair_twist_dft<C, 0>(v, t, tw);
-        // (the previous tile's barrier before its store: the exchange buffer has been read)
-        pair_scatter<C, 0>(v, smem4, pr * C::N, t);
+        // (a thread without a tile skips what no other thread waits for)
+        if (!C::kSteal || tile >= 0) {
+            in_a = sig < batch, in_b = sig + 1 < batch;
+            ea = in_a ? (int)in_exp[sig] : 0, eb = in_b ? (int)in_exp[sig + 1] : 0;
+            const uint32_t* src =
+                reinterpret_cast<const uint32_t*>(base8 + C::kExchangeBytes + slot * C::kSlotBytes) + 2 * pr * C::N;
+            pair_load<C, INV>(v, src, t);
+            pair_twist_dft<C, 0>(v, t, tw);
+            // (the previous tile's barrier before its store: the exchange buffer has been read)
+            pair_scatter<C, 0>(v, smem4, pr * C::N, t);
+        }
         fence_proxy_async_smem();
         // ... and every thread has read the slot: refill it
         if constexpr (C::kSteal) {
-            if (__syncthreads_or(dead)) break;
+            // every thread leaves in the same iteration, also when one gave up
+            if (__syncthreads_or(dead) || tile < 0) break;
             if (tid == 0) {
                 bool late = false;
                 const int64_t next = taker.take(wait_ns, late);

@@ -18,7 +18,9 @@ from tests.helpers import oracle_max_rel_l2
 from tests.test_bank_model import _rows
 from tests.test_bounded_waits import CSRC, blank, function_spans
 
-KERNELS = [("fft_device.cuh", "fft_stockham_slot_ring_kernel")]
+KERNELS = [("fft_device.cuh", "fft_stockham_slot_ring_kernel"), ("fft_device.cuh", "fft_small_steal_kernel"),
+           ("fft_device.cuh", "fft_small_c32_steal_kernel"), ("fft_pair.cuh", "fft_pair_c32_warp_kernel"),
+           ("fft_pair.cuh", "fft_pair_c32_ring_kernel")]
 TOGETHER = r"__sync\w+|__shfl\w+|__any_sync|__reduce_\w+|\bpair_stages\b|\btwist_and_dft\b|\btc_norm_\w+\b"
 UNIFORM = r"__any_sync|__syncthreads_or|C::kStage0Together"  # conditions all threads of a warp or block share
 
