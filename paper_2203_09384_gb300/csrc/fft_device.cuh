@@ -1568,8 +1568,8 @@ __global__ void __launch_bounds__(SC::NT) fft_small_kernel(const float2* in, flo
 }
 
 // The same with one warp per block, taking the tiles of unstarted blocks; the
-// request for the next tile runs behind the current one.  (`tw` and `stall` are
-// accepted so that the host launches it like the longer lengths' kernels.)
+// request for the next tile runs behind the current one.  (`tw` is accepted so
+// that the host launches it like the longer lengths' kernels.)
 template <class SC, bool INV>
 __global__ void __launch_bounds__(SC::NT)
     fft_small_steal_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw, float scale,
@@ -1583,9 +1583,11 @@ __global__ void __launch_bounds__(SC::NT)
         taker.bar = reinterpret_cast<uint64_t*>(steal + 16);
         mbar_init(taker.bar, 1);
         fence_mbar_init();
+        // failure-detection test mode: a phase nothing completes, before any request
+        if (stall && !mbar_wait_bounded(taker.bar, 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         taker.request();
     }
-    for (int64_t tile = blockIdx.x; tile >= 0;) {
+    for (int64_t tile = stall ? -1 : (int64_t)blockIdx.x; tile >= 0;) {
         small_tile<SC, INV>(in, out, batch, scale, smem4, tile);
         if (threadIdx.x == 0) {
             bool late = false;
@@ -1595,7 +1597,7 @@ __global__ void __launch_bounds__(SC::NT)
         }
         tile = __shfl_sync(0xffffffffu, tile, 0);
     }
-    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up
+    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up, or test mode
 }
 
 // ---------------------------------------------------------------------------
@@ -1878,9 +1880,11 @@ __global__ void __launch_bounds__(SC::NT)
         taker.bar = reinterpret_cast<uint64_t*>(steal + 16);
         mbar_init(taker.bar, 1);
         fence_mbar_init();
+        // failure-detection test mode: a phase nothing completes, before any request
+        if (stall && !mbar_wait_bounded(taker.bar, 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         taker.request();
     }
-    for (int64_t tile = blockIdx.x; tile >= 0;) {
+    for (int64_t tile = stall ? -1 : (int64_t)blockIdx.x; tile >= 0;) {
         small_c32_tile<SC, INV>(in, in_exp, out, out_exp, batch, ls, smem4, tile);
         if (threadIdx.x == 0) {
             bool late = false;
@@ -1890,7 +1894,7 @@ __global__ void __launch_bounds__(SC::NT)
         }
         tile = __shfl_sync(0xffffffffu, tile, 0);
     }
-    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up
+    if (threadIdx.x == 0) taker.drain(wait_ns);  // an answer still under way after a wait gave up, or test mode
 }
 
 template <int LOG2N, int WARPS, int U = 1, int CH_ = 0>
