@@ -330,8 +330,9 @@ GBFFT_API fft_status_t fft_validate(int64_t n, int64_t batch, int direction, int
  *  - The first call on a device does a one-time set-up (it looks up the
  *    static array's device address with cudaGetSymbolAddress while that
  *    device is current); the first call for each length, direction and
- *    variant also queries its launch shape.  Make those first calls before
- *    any stream capture.
+ *    variant also queries its launch shape (a call that names no variant: the
+ *    shapes of the schedules for every batch size of that length).  Make those
+ *    first calls before any stream capture.
  *  - Every call enqueues two kernels on `stream`: one rewrites the shared
  *    array (this length's twiddles, error word cleared), one transforms.  All
  *    calls on a device share the array, which keeps the last call's

@@ -200,6 +200,15 @@ extern "C" fft_status_t fft_execute_noalloc(int64_t n, int64_t batch, int direct
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         st = setup_device(dev, &d);
+        // A call that names no variant sets up the kernels of every size of the
+        // length: a later size must not load code (device memory) or query a
+        // launch shape under capture that an earlier call could have prepared.
+        if (variant < 0) {
+            const gbfft::KernelEntry* all[GBFFT_MAX_VARIANTS];
+            const int count = gbfft::default_entries(log2n, all);
+            for (int i = 0; i < count; ++i)
+                if (st == FFT_OK) st = kernel_shape(d, all[i], inverse, &per_sm);
+        }
         if (st == FFT_OK) st = kernel_shape(d, e, inverse, &per_sm);
     }
     if (st != FFT_OK) return st;

@@ -60,18 +60,18 @@ LengthVariants* registry() {
 }
 
 // The variant of a plan that names none: type `tc` (0 FP32, 1 FP16 / 2 BF16
-// tensor cores, 3 complex32), calls of `elems` elements.  Without `steal`, the last row for
-// smaller calls in place of one that needs a block per tile.
+// tensor cores, 3 complex32), calls of `elems` elements.  Without `steal`, the
+// last row for smaller calls in place of one that needs a block per tile.
 constexpr int kTcC32 = 3;
-int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
-    struct Row {
-        int log2n, tc;
-        int64_t max_elems;
-        int variant;
-    };
+struct SizeDefault {
+    int log2n, tc;
+    int64_t max_elems;
+    int variant;
+};
 #define GBFFT_DX(L, TC, MAX, V) {L, TC, MAX, V},
-    static constexpr Row kRows[] = {GBFFT_SIZE_DEFAULTS(GBFFT_DX)};
+constexpr SizeDefault kSizeDefaults[] = {GBFFT_SIZE_DEFAULTS(GBFFT_DX)};
 #undef GBFFT_DX
+int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
     const LengthVariants& lv = registry()[log2n];
     int fallback = 0;
     if (tc == kTcC32) {
@@ -82,7 +82,7 @@ int default_variant(int log2n, int tc, int64_t elems, bool steal = true) {
     } else if (const int preferred = lv.preferred.load()) {
         return preferred;
     }
-    for (const Row& r : kRows) {
+    for (const SizeDefault& r : kSizeDefaults) {
         if (r.log2n != log2n || r.tc != tc || (!steal && lv.v[r.variant].steal)) continue;
         if (elems <= r.max_elems) return r.variant;
         if (!steal) fallback = r.variant;
@@ -167,6 +167,16 @@ const KernelEntry* lookup_entry(int log2n, int variant, int64_t elems) {
     if (variant < 0) variant = default_variant(log2n, 0, elems);
     if (variant >= lv->count || !lv->v[variant].kernel_fwd) return nullptr;
     return &lv->v[variant];
+}
+
+int default_entries(int log2n, const KernelEntry** out) {
+    const LengthVariants& lv = registry()[log2n];
+    const int preferred = lv.preferred.load();
+    int count = 0;
+    out[count++] = &lv.v[preferred];
+    for (const SizeDefault& r : kSizeDefaults)
+        if (!preferred && r.log2n == log2n && r.tc == 0) out[count++] = &lv.v[r.variant];
+    return count;
 }
 }  // namespace gbfft
 

@@ -55,6 +55,9 @@ cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, voi
 // Registry lookup (host): the entry of `variant`, or when variant < 0 of the
 // FP32 default for calls of `elems` elements; NULL when there is none.
 const KernelEntry* lookup_entry(int log2n, int variant, int64_t elems);
+// Every entry that lookup_entry may give for variant < 0 at some size (up to
+// GBFFT_MAX_VARIANTS of them, with repeats); returns how many.
+int default_entries(int log2n, const KernelEntry** out);
 
 // Ragged (mixed-length) plans, implemented in fft_ragged.cu.
 struct RaggedState;
