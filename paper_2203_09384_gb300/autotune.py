@@ -64,10 +64,23 @@ def _time(fn, reps: int, warmup: int = 2) -> float:
     return statistics.median(ts)
 
 
+def _plan_by_size(n: int, batch: int, device):
+    """A plan as a default of 0 gives it, whatever the current default is."""
+    from . import Plan
+    before = _abi.fft_get_default_variant(n)
+    _abi.fft_set_default_variant(n, 0)
+    try:
+        return Plan(n, batch, device=device)
+    finally:
+        _abi.fft_set_default_variant(n, before)
+
+
 def tune_lengths(lengths=LENGTHS, elems: int = 2 ** 26, reps: int = 7, apply: bool = True,
                  device=None) -> dict:
     """Time every variant of every length on `elems` complex64 elements
-    (uniform [-1, 1]); returns {n: {"best": v, "ms": {v: ms}}}."""
+    (uniform [-1, 1]); returns {n: {"best": v, "ms": {v: ms}}}.  Number 0 stands
+    for what a default of 0 runs, the compiled schedule for the size of the
+    call, and is timed as such."""
     from . import Plan
     dev = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
     g = torch.Generator(device=dev)
@@ -81,7 +94,7 @@ def tune_lengths(lengths=LENGTHS, elems: int = 2 ** 26, reps: int = 7, apply: bo
         for v in range(_abi.fft_variant_count(n)):
             if _abi.fft_variant_dtype(n, v) != _abi.FFT_C64:
                 continue  # tensor-core variants are chosen by dtype, not tuned against FP32
-            p = Plan(n, elems // n, variant=v, device=dev)
+            p = Plan(n, elems // n, variant=v, device=dev) if v else _plan_by_size(n, elems // n, dev)
             timings[v] = _time(lambda: p.execute(x, out), reps)
             if p.error() != 0:
                 timings[v] = float("inf")
