@@ -7,6 +7,8 @@ import paper_2203_09384_gb300 as gb
 from paper_2203_09384_gb300 import _abi, autotune
 
 N = 256
+FP32 = [v for v in range(_abi.fft_variant_count(N)) if _abi.fft_variant_dtype(N, v) == _abi.FFT_C64]
+OTHER = FP32[1]
 
 
 @pytest.fixture
@@ -34,13 +36,12 @@ def made(monkeypatch):
 
 
 def test_zero_is_timed_by_size(made):
-    _abi.fft_set_default_variant(N, 1)
+    _abi.fft_set_default_variant(N, OTHER)
     result = autotune.tune_lengths([N], elems=1 << 12, apply=False, device="cpu")
     assert made[0] == (None, 0)
-    fp32 = [v for v in range(_abi.fft_variant_count(N)) if _abi.fft_variant_dtype(N, v) == _abi.FFT_C64]
-    assert [v for v, _ in made[1:]] == fp32[1:] and all(d == 1 for _, d in made[1:])
-    assert result[N]["best"] == 0 and sorted(result[N]["ms"]) == fp32
-    assert _abi.fft_get_default_variant(N) == 1
+    assert [v for v, _ in made[1:]] == FP32[1:] and all(d == OTHER for _, d in made[1:])
+    assert result[N]["best"] == 0 and sorted(result[N]["ms"]) == FP32
+    assert _abi.fft_get_default_variant(N) == OTHER
     autotune.tune_lengths([N], elems=1 << 12, device="cpu")
     assert _abi.fft_get_default_variant(N) == 0
 
@@ -50,7 +51,7 @@ def test_a_plan_that_cannot_be_made_leaves_the_default(made, monkeypatch):
         raise RuntimeError
 
     monkeypatch.setattr(gb, "Plan", broken)
-    _abi.fft_set_default_variant(N, 1)
+    _abi.fft_set_default_variant(N, OTHER)
     with pytest.raises(RuntimeError):
         autotune.tune_lengths([N], elems=1 << 12, device="cpu")
-    assert _abi.fft_get_default_variant(N) == 1
+    assert _abi.fft_get_default_variant(N) == OTHER
