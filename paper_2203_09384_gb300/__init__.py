@@ -75,9 +75,11 @@ def _stored(t: torch.Tensor, stream=None) -> torch.Tensor:
 
 
 # The two queries every call needs, without the wrappers' device objects,
-# context managers and stream objects (together about 4 us a call).
-_current_device = torch._C._cuda_getDevice
-_current_raw_stream = torch._C._cuda_getCurrentRawStream
+# context managers and stream objects (together about 4 us a call); the
+# wrappers where a build of torch does not have the names behind them.
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
+                              lambda index: torch.cuda.current_stream(index).cuda_stream)
 
 
 def _enqueue(index: int, stream, call, *args) -> None:
