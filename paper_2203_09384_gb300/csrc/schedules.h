@@ -121,7 +121,8 @@
     GX(10, 18, 16, 2, 8, 16, 8, 0, 6, 2, 2, -3, 6) \
     GX(11, 20, 16, 1, 16, 8, 16, 0, 3, 2, 0, -1, 2) \
     GX(11, 21, 16, 1, 8, 16, 16, 0, 5, 2, 1, -3, 6) \
-    GX(11, 22, 16, 1, 8, 16, 16, 0, 5, 2, 2, -3, 6)
+    GX(11, 22, 16, 1, 8, 16, 16, 0, 5, 2, 2, -3, 6) \
+    GX(11, 24, 16, 1, 16, 8, 16, 0, 3, 0, 0, 0, 0)
 
 #define GBFFT_SMALL_SCHEDULES(SX) \
     SX(1, 0, 1, 8, 4)                \
@@ -203,8 +204,8 @@
 // the last one, variant 0 (FP32) or the first variant of the type.  A default
 // set by fft_set_default_variant (the autotuner's) goes before all of this.
 //
-// Past some 6 M elements the rows that take tiles of unstarted blocks (CH bit 2)
-// win: variant 0 at every length.  Their first request costs about 1 us, so
+// Past some 6 M elements (N = 2048: 12 M) the rows that take tiles of unstarted
+// blocks (CH bit 2) win: variant 0 at every length.  Their first request costs about 1 us, so
 // shorter calls run fixed strides, and with few tiles per SM want small blocks
 // and tiles, which start their first store sooner and leave a shorter tail;
 // evict-first direct loads and stores win while the output still fits in L2.
@@ -222,6 +223,12 @@
 //   N = 512   2^21.4 12.1 /  8.7 /  -     2^22.2 16.2 / 14.4 / 15.4   2^24 45.2 / 43.4 / 41.9   2^28 636 / 603
 //   N = 1024  2^21.4 11.8 /  9.0 /  -     2^22.2 17.3 / 15.5 / 16.4   2^24 45.6 / 43.4 / 41.9   2^28 650 / 602
 //   N = 2048  2^21.4 12.0 /  9.8 / 12.9   2^23.2 28.7 / 27.4 / 28.0   2^24 45.7 / 44.5 / 44.0   2^28 652 / 607
+// All rows of a length take its radices in one order, so a signal's result does
+// not depend on how many others share its call.  At N = 2048 the ring (20) and
+// the direct row (24) cross four times, as one more block an SM costs the one a
+// round and the other less; ring / direct, calls chained in a graph: 602 K
+// elements (294 signals) 2.9 / 3.2, 645 K 4.2 / 3.2, 2^20 4.3 / 4.0, 2^20.1 4.4 /
+// 4.6, 2^20.5 5.7 / 5.8, 2^20.6 6.4 / 5.9, 2^20.9 7.7 / 7.5, 2^21 8.1 / 8.5.
 // The rows up to 2^16 and 2^17 of N = 64 and 128 keep those plans on bulk-copy
 // kernels (0.3-0.8 us over the direct rows, 0.4 under the earlier default).
 //
@@ -250,8 +257,10 @@
     DX(10, 0, 1 << 20, 16)      \
     DX(10, 0, 5 << 20, 15)      \
     DX(10, 0, 7 << 20, 16)      \
-    DX(11, 0, 3 << 19, 20)      \
-    DX(11, 0, 3 << 20, 1)       \
+    DX(11, 0, 5 << 17, 20)      \
+    DX(11, 0, 1 << 20, 24)      \
+    DX(11, 0, 23 << 16, 20)     \
+    DX(11, 0, 15 << 17, 24)     \
     DX(11, 0, 12 << 20, 20)     \
     DX(7, 1, 2 << 20, 1)        \
     DX(7, 1, 16 << 20, 9)       \
