@@ -108,7 +108,7 @@ static KernelEntry c32_row(int variant) {
         return pair_c32_entry<PairCfg<L, E, S, R0, R1, R2, R3, MINB, PIPE, (XB & 8) != 0>>(variant);
     } else {
         static_assert(PIPE == 0, "one signal per thread group: direct loads");
-        return c32_entry<Cfg<L, E, S, R0, R1, R2, R3, MINB, 0, 0, XB, 0>>(variant);
+        return c32_entry<Cfg<L, E, S, R0, R1, R2, R3, MINB, 0, 0, XB, 8>>(variant);
     }
 }
 
