@@ -1804,8 +1804,8 @@ struct C32Smem {
     static constexpr int kBytes = kRedOffset + 128;
 };
 
-// Direct loads (the N <= 32 rows beside the one-thread-per-signal defaults;
-// N = 64..2048: fft_pair.cuh).  err / wait_ns / stall are accepted so that all
+// Direct loads (the N <= 32 rows beside the one-thread-per-signal defaults, and
+// short calls of N = 256, 1024 and 2048; else N = 64..2048: fft_pair.cuh).  err / wait_ns / stall are accepted so that all
 // complex32 kernels share one argument list; nothing here waits.
 template <class C, bool INV>
 __global__ void __launch_bounds__(C::NT, C::MINB)

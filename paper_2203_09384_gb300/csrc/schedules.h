@@ -151,7 +151,8 @@
 // (fft_pair.cuh), S / 2 signal pairs and S N / (2 E) threads per block, a ring
 // of PIPE bulk-copied tiles per warp (N <= 512) or per block; XB = 14: the same,
 // taking the tiles of unstarted blocks (one warp per block for N <= 512).  XB = 0: the
-// Stockham kernel with binary16 loads/stores, one signal per thread group.
+// Stockham kernel with binary16 loads/stores, one signal per thread group (N >= 64:
+// in the pair kernels' arithmetic, bit for bit).
 // A length's first complex32 row is its default; for N <= 32 that is the
 // one-thread-per-signal SCX row further down.
 //
@@ -172,12 +173,12 @@
     CX(6, 1, 16, 64, 8, 8, 0, 0, 4, 1, 6)        \
     CX(7, 5, 16, 32, 8, 16, 0, 0, 4, 1, 6)       \
     CX(8, 18, 16, 8, 16, 16, 0, 0, 8, 1, 6)      \
-    CX(8, 6, 16, 16, 16, 16, 0, 0, 3, 2, 6)      \
+    CX(8, 6, 16, 4, 16, 16, 0, 0, 1, 0, 0)       \
     CX(9, 2, 16, 8, 8, 8, 8, 0, 4, 1, 6)         \
     CX(10, 8, 16, 2, 8, 16, 8, 0, 8, 1, 6)       \
-    CX(10, 9, 16, 4, 8, 16, 8, 0, 4, 1, 6)       \
+    CX(10, 9, 16, 1, 8, 16, 8, 0, 4, 0, 0)       \
     CX(11, 8, 16, 2, 8, 16, 16, 0, 4, 1, 6)      \
-    CX(11, 9, 16, 2, 8, 16, 16, 0, 3, 2, 6)      \
+    CX(11, 9, 16, 1, 8, 16, 16, 0, 3, 0, 0)      \
     CX(8, 5, 16, 16, 16, 16, 0, 0, 4, 1, 6)      \
     CX(6, 7, 16, 16, 8, 8, 0, 0, 16, 1, 14)      \
     CX(7, 13, 16, 8, 8, 16, 0, 0, 16, 1, 14)     \
@@ -241,7 +242,14 @@
 // complex32 (type 3), us, fixed stride / taken tiles: N = 4 2^24 26.2 / 23.8, 8
 // 2^27 179 / 163, 16 2^27 174 / 158, 32 2^27 165 / 160, 64 2^27 169 / 164, 128
 // 2^27 178 / 169, 256 2^27 181 / 169, 1024 2^27 218 / 213, 2048 2^27 240 / 232;
-// N = 2 (211 / 237) and N = 512 (208 / 208) keep the fixed stride.
+// N = 2 (211 / 237) and N = 512 (208 / 208) keep the fixed stride.  Short calls of
+// N = 256, 1024 and 2048 take one signal per thread group and blocks of 64 or
+// 128 threads: a thread's chain is shorter, and the machine is not full anyway.
+// Two signals per thread / one, calls chained in a graph, us: N = 256 2^12 2.2 /
+// 1.55, 2^18 2.4 / 1.8, 2^20 3.3 / 2.9, 2^20.5 4.7 / 3.9, 2^21.25 5.2 / 5.1, 2^21.5
+// 6.2 / 6.6; N = 1024 2^12 2.4 / 1.8, 2^18 2.75 / 2.2, 2^19 3.0 / 2.7, 588 signals
+// 3.05 / 2.85, 630 (over four blocks an SM) 3.2 / 3.35; N = 2048 2^12 2.7 / 1.9,
+// 2^18 2.9 / 2.1, 222 signals 3.0 / 2.7, 238 3.05 / 3.3.
 #define GBFFT_SIZE_DEFAULTS(DX) \
     DX(1, 0, 5 << 20, 4)        \
     DX(2, 0, 5 << 20, 6)        \
@@ -292,11 +300,13 @@
     DX(6, 3, INT64_MAX, 7)      \
     DX(7, 3, 14 << 20, 5)       \
     DX(7, 3, INT64_MAX, 13)     \
-    DX(8, 3, 1 << 19, 18)       \
+    DX(8, 3, 5 << 19, 6)        \
     DX(8, 3, 12 << 20, 5)       \
     DX(8, 3, INT64_MAX, 24)     \
+    DX(10, 3, 19 << 15, 9)      \
     DX(10, 3, 48 << 20, 8)      \
     DX(10, 3, INT64_MAX, 19)    \
+    DX(11, 3, 7 << 16, 9)       \
     DX(11, 3, 20 << 20, 8)      \
     DX(11, 3, INT64_MAX, 23)
 
