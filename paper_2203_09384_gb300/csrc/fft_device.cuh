@@ -328,9 +328,9 @@ __device__ __forceinline__ int swz16(int a) {
 
 // Programmatic dependent launch.  Every kernel here starts with pdl_enter():
 // it waits until the previous kernel of the stream has completed and its
-// memory is visible, before touching any buffer, then lets the next kernel
-// launch (so that its blocks are scheduled while this grid runs and drains,
-// instead of after it).  Both steps are no-ops for a kernel launched without
+// memory is visible, before touching any buffer.  pdl_release() then lets the
+// next kernel launch (so that its blocks are scheduled while this grid runs and
+// drains, instead of after it).  Both are no-ops for a kernel launched without
 // programmatic stream serialization.
 //
 // In this order one waiting grid at most shares the device with the running
@@ -340,8 +340,17 @@ __device__ __forceinline__ int swz16(int a) {
 // plain / released first / in this order, us: 2^18 elements of N = 2 2.04 / 2.41
 // / 1.87, N = 256 2.53 / 3.10 / 2.16, N = 2048 2.64 / 3.84 / 2.26; 2^20 of N = 256
 // 4.29 / 3.91 / 3.89; the smallest calls 1.91 / 1.48 / 1.59 (2^10 of N = 256).
+//
+// Most kernels release right after the wait.  Where a grid that fills the
+// device lost 0.2-0.4 us a call by that against the release before the wait,
+// the release stands behind the first loads: released first / right after the
+// wait / behind the first loads, 1000003 signals of N = 8 20.7 / 21.0 / 20.6 us,
+// complex32 100003 of N = 128 21.0 / 21.2 / 20.7 (there behind the first tile;
+// behind its loads alone 21.2).
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_release() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
@@ -1229,6 +1238,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw, float scale,
                         int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     extern __shared__ __align__(16) float2 smem[];
     const int tid = threadIdx.x;
     const int sl = tid / C::T;
@@ -1282,6 +1292,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_ring_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw,
                              float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     constexpr int D = C::PIPE;
     constexpr int TILE = C::S * C::N;
     extern __shared__ __align__(16) float2 smem[];
@@ -1400,6 +1411,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_slot_ring_kernel(const float2* in, float2* out, int64_t batch, const float2* __restrict__ tw,
                                   float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     static_assert(C::kInRing, "in-ring schedules only");
     constexpr int D = C::PIPE;
     constexpr int TILE = C::kSlotElems;
@@ -1626,6 +1638,7 @@ template <class SC, bool INV>
 __global__ void __launch_bounds__(SC::NT) fft_small_kernel(const float2* in, float2* out, int64_t batch,
                                                            float scale) {
     pdl_enter();
+    pdl_release();
     constexpr int W = SC::WARPS_PER_BLOCK, TS = 32 * SC::UNROLL;
     extern __shared__ __align__(16) float4 smem4[];
     const int warp = threadIdx.x >> 5;
@@ -1654,6 +1667,7 @@ __global__ void __launch_bounds__(SC::NT)
         if (stall && !mbar_wait_bounded(taker.bar, 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         taker.request();
     }
+    pdl_release();
     for (int64_t tile = stall ? -1 : (int64_t)blockIdx.x; tile >= 0;) {
         small_tile<SC, INV>(in, out, batch, scale, smem4, tile);
         if (threadIdx.x == 0) {
@@ -1812,6 +1826,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_stockham_c32_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp, int64_t batch,
                             const float2* __restrict__ tw, float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     extern __shared__ __align__(16) float2 smem[];
     float* red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(smem) + C32Smem<C>::kRedOffset);
     const int tid = threadIdx.x;
@@ -1922,6 +1937,7 @@ __global__ void __launch_bounds__(SC::NT)
     fft_small_c32_kernel(const __half2* in, const int8_t* in_exp, __half2* out, int8_t* out_exp, int64_t batch,
                          const float2* __restrict__ tw, float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     constexpr int W = SC::WARPS_PER_BLOCK, TS = 32 * SC::UNROLL, P = TS * SC::N / 4;
     extern __shared__ __align__(16) float4 smem4[];
     const int warp = threadIdx.x >> 5;
@@ -1951,6 +1967,7 @@ __global__ void __launch_bounds__(SC::NT)
         if (stall && !mbar_wait_bounded(taker.bar, 0, wait_ns)) atomicCAS(err, 0, kErrTimeout);
         taker.request();
     }
+    pdl_release();
     for (int64_t tile = stall ? -1 : (int64_t)blockIdx.x; tile >= 0;) {
         small_c32_tile<SC, INV>(in, in_exp, out, out_exp, batch, ls, smem4, tile);
         if (threadIdx.x == 0) {

@@ -517,6 +517,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
         }
         pair_twist_dft<C, 0>(v, t, tw);
         pair_stages<C, 1>(v, xbuf, pr * C::N, t, tw);
+        if (tile == first_tile) pdl_release();
         const float2 m = pair_max<C>(v);
         const C32Out oa = c32_out_scale<C::N>(m.x, ea, ls), ob = c32_out_scale<C::N>(m.y, eb, ls);
         const bool warp_dead = __any_sync(0xffffffffu, dead);
@@ -560,6 +561,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     fft_pair_c32_ring_kernel(const uint32_t* in, const int8_t* in_exp, uint32_t* out, int8_t* out_exp, int64_t batch,
                              const float2* __restrict__ tw, float scale, int* err, uint64_t wait_ns, int stall) {
     pdl_enter();
+    pdl_release();
     constexpr int D = C::D;
     extern __shared__ __align__(16) float4 smem4[];
     unsigned char* base8 = reinterpret_cast<unsigned char*>(smem4);

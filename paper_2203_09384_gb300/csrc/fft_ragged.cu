@@ -264,6 +264,7 @@ __device__ __forceinline__ void ragged_dispatch(const RaggedArgs& a, const Ragge
 template <int V, bool INV>
 __global__ void __launch_bounds__(kRaggedThreads, RaggedMinBlocks<V & 1>::value) fft_ragged_kernel(RaggedArgs a) {
     pdl_enter();
+    pdl_release();
     constexpr int S = V & 1;  // schedule set
     extern __shared__ __align__(16) float2 smem[];
     dbg_set_err(a.err);
@@ -348,6 +349,7 @@ __device__ __forceinline__ void ragged_ring_tile(const RaggedArgs& a, const Ragg
 template <bool INV>
 __global__ void __launch_bounds__(kRaggedThreads, 3) fft_ragged_ring_kernel(RaggedArgs a) {
     pdl_enter();
+    pdl_release();
     extern __shared__ __align__(16) float2 smem[];
     float2* xbuf = smem;                   // 2 exchange buffers
     float2* ring = smem + 2 * kRingTile;   // 2 ring slots
@@ -570,7 +572,8 @@ __device__ __forceinline__ void slot_tile(const RaggedArgs& a, const RaggedItem&
 // descriptor is loaded before the wait for a free slot, and the offsets of a
 // tile of scattered signals after the copies of the item before, so that their
 // latency hides behind that wait.  A back-to-back tile's first signal comes
-// with its own offset (RaggedItem::off0).  Before it exits, lane 0 waits (bounded) for the copies it issued last, so none
+// with its own offset (RaggedItem::off0).  Before it exits, lane 0 waits
+// (bounded) for the copies it issued last, so none
 // lands after the block is gone even when the compute threads gave up.
 template <int NTC, int SLOTS, int MINB>
 __device__ __forceinline__ void slot_produce(const RaggedArgs& a, float2* ring, uint64_t* full, uint64_t* empty,
@@ -710,6 +713,7 @@ template <int NTC, int SLOTS, int MINB, bool INV>
 __global__ void __launch_bounds__(SlotShape<NTC, MINB>::kThreads, SlotShape<NTC, MINB>::kMinBlocks)
     fft_ragged_slot_kernel(RaggedArgs a) {
     pdl_enter();
+    pdl_release();
     ragged_slot_body<NTC, SLOTS, MINB, 0, INV>(a);
 }
 
@@ -720,6 +724,7 @@ __global__ void __launch_bounds__(SlotShape<NTC, MINB>::kThreads, SlotShape<NTC,
 template <int NTC, int SLOTS, int REGS, int CH, bool INV>
 __global__ void __maxnreg__(REGS) fft_ragged_slot_kernel_capped(RaggedArgs a) {
     pdl_enter();
+    pdl_release();
     ragged_slot_body<NTC, SLOTS, 5, CH, INV>(a);
 }
 

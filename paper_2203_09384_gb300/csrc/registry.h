@@ -44,11 +44,12 @@ struct KernelEntry {
 void begin_plan_allocs();
 cudaError_t plan_malloc(void** ptr, size_t bytes);
 // Every kernel launch of the library but fft_execute_noalloc's: with
-// programmatic stream serialization (unless the caller declines it), so that the kernel may be scheduled while the previous
-// kernel of the stream drains (each kernel waits for its predecessor before
-// touching memory, pdl_enter).  Small calls gain most: back to back through the
-// Python binding 2^20 elements of N = 256 6.1 -> 3.9 us, 2^21 of N = 1024 10.3
-// -> 9.1, 2^10 3.8-4.1 -> 3.6-3.8 (the extended launch costs the host no more).
+// programmatic stream serialization (unless the caller declines it), so that
+// the kernel may be scheduled while the previous kernel of the stream drains
+// (each kernel waits for its predecessor before touching memory, pdl_enter).
+// Small calls gain most: back to back through the Python binding 2^20 elements
+// of N = 256 6.1 -> 3.9 us, 2^21 of N = 1024 10.3 -> 9.1, 2^10 3.8-4.1 -> 3.6-3.8
+// (the extended launch costs the host no more).
 cudaError_t launch_kernel(const void* kernel, unsigned grid, unsigned block, void** args, size_t smem,
                           cudaStream_t stream, bool programmatic = true);
 
