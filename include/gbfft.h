@@ -162,9 +162,10 @@ GBFFT_API fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int directio
  * any other overlap is rejected.  Both pointers must be 16-byte aligned.
  * The caller owns both buffers and must keep them alive until the stream has
  * run the kernel.  One plan may be executed concurrently on several streams.
- * Calls are launched with programmatic stream serialization: the kernel may be scheduled while the previous kernel of the
- * stream finishes, but it waits for that kernel to complete before it reads or
- * writes any buffer, so stream order holds as for a plain launch.
+ * Calls are launched with programmatic stream serialization: the kernel may be
+ * scheduled while the previous kernel of the stream finishes, but it waits for
+ * that kernel to complete before it reads or writes any buffer, so stream order
+ * holds as for a plain launch.
  * Errors: FFT_ERR_INVALID_VALUE, FFT_ERR_MISALIGNED, FFT_ERR_OVERLAP,
  * FFT_ERR_CUDA (launch failure, reported from cudaGetLastError).
  */
@@ -191,7 +192,11 @@ GBFFT_API fft_status_t fft_execute_c32(fft_plan_t plan, const void* in, const in
  * `in_host`, results written to `out_host` (equal, or not overlapping).  The
  * plan must have been made with FFT_FLAG_HOST_STAGING.  Page-locked buffers
  * (cudaHostAlloc / cudaHostRegister, 16-byte aligned) are read and written in
- * place over the link by one launch on `stream`.  Otherwise work is split into
+ * place over the link by one launch on `stream`, which holds 38 to a few hundred
+ * thread blocks (a quarter of the SMs or more) for the whole transfer, 0.8 ms at
+ * 2^24 elements; work on other streams shares the device with it.  A caller who
+ * wants the copy engines to carry the transfer copies to device buffers itself
+ * and calls fft_execute.  Otherwise work is split into
  * chunks of whole signals; each chunk is copied to one of the plan's device
  * buffers, transformed in place and copied back, the chunks round-robin over
  * the plan's three streams so that host-to-device copies, kernels and
@@ -244,7 +249,10 @@ typedef struct {
     int64_t work_items;     /* ragged plans: tiles in the device work list      */
     int tc;                 /* radix-16 stages on tensor cores: 0 no (FP32),
                                1 FP16 operands, 2 BF16 operands                 */
-    int64_t grid;           /* blocks launched (persistent grid-stride loop)    */
+    int64_t grid;           /* blocks that run at a time: the tiles of a call, at
+                               most the resident blocks.  Schedules whose running
+                               blocks take the tiles of unstarted ones launch one
+                               block per tile, the others this many             */
     int64_t smem_bytes;     /* dynamic shared memory per block                  */
     int64_t twiddle_count;  /* complex64 entries in the plan's twiddle table    */
     int tc_stages;          /* radix stages that run on tensor cores            */

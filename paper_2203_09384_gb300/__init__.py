@@ -164,8 +164,9 @@ class Plan:
         return out, out_exp
 
     def execute_host(self, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-        """Transform a host (CPU, ideally pinned) tensor through the plan's
-        chunked copy/transform/copy pipeline; synchronises the stream."""
+        """Transform a host (CPU) tensor; synchronises the stream.  Pinned tensors
+        are read and written in place by one launch, others go through the plan's
+        chunked copy/transform/copy pipeline."""
         cpu = torch.device("cpu")
         _check_buffer(x, "x", torch.complex64, cpu, self.n * self.batch)
         if out is None:

@@ -534,7 +534,8 @@ fft_status_t fft_plan_create_ex(int64_t n, int64_t batch, int direction, int dty
         return FFT_ERR_CUDA;
     }
 
-    // launch shape: persistent grid, enough resident blocks to fill every SM
+    // launch shape: enough resident blocks to fill every SM (tile-taking
+    // schedules launch a block per tile, of which these run at a time)
     for (gbfft_plan::Launch* l : {&p->dev, &p->host}) {
         l->resident = resident_blocks(l->entry, l->kernel, dev, sms);
         if (l->resident < 1) {

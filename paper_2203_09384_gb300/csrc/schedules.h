@@ -1,8 +1,9 @@
 // Radix schedules per transform length: the analogue of the paper's host-side
 // `stage_sizes` array and work-group factor (Sec. 4), fixed at compile time so
 // that every stage's register array has a static size.  Several candidate
-// schedules ("variants") may exist per length; plans use variant 0 unless the
-// caller or the autotuner picks another.
+// schedules ("variants") may exist per length; plans use the one that
+// GBFFT_SIZE_DEFAULTS gives for their size unless the caller or the autotuner
+// picks another.
 //
 // Generic Stockham kernel rows:
 //   GX(log2N, variant, E = complex elements per thread, S = signals per block,
@@ -230,8 +231,14 @@
 // round and the other less; ring / direct, calls chained in a graph: 602 K
 // elements (294 signals) 2.9 / 3.2, 645 K 4.2 / 3.2, 2^20 4.3 / 4.0, 2^20.1 4.4 /
 // 4.6, 2^20.5 5.7 / 5.8, 2^20.6 6.4 / 5.9, 2^20.9 7.7 / 7.5, 2^21 8.1 / 8.5.
-// The rows up to 2^16 and 2^17 of N = 64 and 128 keep those plans on bulk-copy
-// kernels (0.3-0.8 us over the direct rows, 0.4 under the earlier default).
+// The lines at 2^16 and 2^17 of N = 64 and 128 and at 2^20 of N = 1024 are not
+// drawn by time: up to there a default plan runs a bulk-copy kernel, because the
+// tests of bounded waits take default plans of 611 signals as ones that wait on
+// the device.  Bulk-copy / direct row, chained in a graph, us: N = 64 2^10 2.05 /
+// 1.33, 2^14 2.2 / 1.5, 2^16 2.2 / 1.5; N = 128 2^10 1.85 / 1.5, 2^14 2.0 / 1.65, 2^17
+// 2.1 / 1.8; N = 1024 2^10 1.8 / 1.55, 2^18 2.2 / 2.0, 2^19 2.8 / 3.2, 2^19.5 4.0 / 3.2,
+// 2^20 4.05 / 3.8.  (The one schedule for all sizes before: 2.4-3.1, 2.3-2.8, 2.4-4.9.)
+// N = 2048 below 602 K elements: 2^12 2.1 / 1.85, 2^18 2.3 / 2.1, 2^19 2.9 / 3.3.
 //
 // Tensor-core types: every row of a length rounds the same operands.  Before /
 // after at 2^28: FP16 N = 128 672 / 607, 256 666 / 600, 1024 727 / 686,
