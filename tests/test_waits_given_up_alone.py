@@ -1,4 +1,4 @@
-"""Every thread judges a bounded wait for itself, so some threads of a block may
+"""Every thread decides a bounded wait for itself, so some threads of a block may
 give up where others do not.  Whatever a warp or a block does together
 (barriers, shuffles, votes, the aligned tensor-core instructions) must then not
 sit under a condition on the thread's own outcome.
